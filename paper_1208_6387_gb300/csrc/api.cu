@@ -13,6 +13,7 @@
 #include "../../include/fetirp.h"
 #include "common.cuh"
 #include "dense.cuh"
+#include "oz.cuh"
 #include "ops.cuh"
 #include "tc.cuh"
 
@@ -90,6 +91,18 @@ __global__ void k_unpermute_rotate(int n_dofs, int dpn, int npad, const double* 
 }
 
 // ------------------------------------------------------------------------------------------- host data
+// Owned scratch of the sliced FP64 products, kept between factorisations.
+struct OzBuf {
+  DBuf<uint8_t> slices;
+  DBuf<int> exps;
+  OzOperand operand(long long rows, long long cols) {
+    slices.ensure((size_t)oz_tiles(rows, cols) * OZ_TILE);
+    exps.ensure((size_t)round_up(rows, 64));
+    return {slices.p, exps.p};
+  }
+  OzOperand operand() const { return {slices.p, exps.p}; }
+};
+
 struct PatternData {
   int n_nodes = 0, dpn = 1, n = 0, n_b = 0, n_i = 0, npad = 0, nbpad = 0, expected = -1, kdim = 0;
   std::vector<int64_t> rowptr;
@@ -100,6 +113,9 @@ struct PatternData {
   DBuf<int64_t> d_rowptr;
   DBuf<int> d_col, d_newidx, zp;
   DBuf<double> d_val, L, diag0, S64, N, Nb, Dinv, LS, XS, DinvS, Sdag, Nwork;
+  // sliced operators of the FP64 local products (n_b >= OZ_LOCAL_MIN_NB): S^+ (with s64_ok), and of a pattern that may
+  // have no formed S^+ the factor Lam = L_S^{-1} and its transpose
+  OzBuf oz_S, oz_lam, oz_lamt;
   DBuf<int> zpS, d_zpiv;
   std::vector<int> h_zp;
   int* h_zp_pinned = nullptr;
@@ -259,6 +275,7 @@ struct fetirp_ctx_s {
   DBuf<double> eta_part;          // row-chunk partials of eta and W^T r
   DBuf<int> n_kept;
   DBuf<double> Y64, Z64, W64;     // W64: scratch of the factored FP64 local product (large patterns)
+  OzBuf oz_rhs;                   // slices of the right-hand sides of the sliced FP64 products
   DBuf<float> Y32, Z32, Ylo32;
   DBuf<float> tc_part;            // K-split partials of the tensor-core product (small blocks only)
   DBuf<int> tc_error;
@@ -433,6 +450,15 @@ bool operator_precision(int p) {
     if (!(cond)) throw Error(FETIRP_EINVAL, msg); \
   } while (0)
 
+// The flag of the bounded tensor-core waits, zeroed on the context's stream.
+void ensure_tc_error(fetirp_ctx ctx) {
+  if (ctx->tc_error.p) return;
+  ctx->tc_error.alloc(1);
+  ctx->tc_error.zero(ctx->stream);
+}
+
+void check_tc_error(fetirp_ctx ctx);
+
 // ----------------------------------------------------------------------------------------- pattern set-up
 // FP64 factorisation on the device: dense factor of K in interior-first/boundary-last order with zero-pivot
 // detection (Sec. 2), kernel N, Schur complement pseudo-inverse S^+ = L_S^{-T} L_S^{-1} (stated after Eq. 3).
@@ -473,6 +499,12 @@ void factor_check(PatternData& P) {
 
 // Patterns with at least this many boundary dofs form S^dag on the tensor cores (factor_stage_b)
 constexpr int TC_SDAG_MIN_NB = 1024;
+// FP64 local products with at least this many boundary dofs and FMAs are sliced tensor-core products (oz.cuh).  Where
+// the line lies (whole apply, FP64 FMAs against sliced, us): n_b 294, 108 right-hand sides (9.3M FMAs) 92 / 103; 654, 32
+// (13.7M) 115 / 118; 1158, 16 (21M) 153 / 148; 456, 108 (22M) 142 / 119; 888, 150 (118M) 333 / 177; 2598, 64 (432M)
+// 1388 / 267; 1158, 1440 (1.9G) 3778 / 428.
+constexpr int OZ_LOCAL_MIN_NB = 256;
+constexpr long long OZ_LOCAL_MIN_FMAS = 1ll << 24;
 void form_splus64(PatternData& P, cudaStream_t s);
 void form_sdag64(PatternData& P, cudaStream_t s);
 
@@ -519,6 +551,7 @@ void factor_stage_b(PatternData& P, int* tc_error, cudaStream_t s) {
   tile_inverses(P.LS.p, nbp, P.zpS.p, P.DinvS.p, s);
   tri_solve(P.LS.p, nbp, P.planS, P.zpS.p, P.XS.p, nbp, nbp, false, s, P.DinvS.p, true);   // X = L_S^{-1}
   const int nb = P.n_b;
+  if (nb >= OZ_LOCAL_MIN_NB) P.oz_S.operand(nb, nb);
   P.lds = round_up(nb, 4);
   P.ldsb = round_up(nb, 8);
   P.ld_y8 = P.ldsb;
@@ -547,6 +580,8 @@ void factor_stage_b(PatternData& P, int* tc_error, cudaStream_t s) {
   // the bf16 pair's own rounding (2^-17), not that of an FP32 rounding, so the FP32 and tf32 forms of S^dag
   // come from the FP64 S^+ (ensure_splus64).
   P.s64_ok = false;
+  oz_slice_cols(P.XS.p, nbp, nb, nb, -1, P.oz_lam.operand(nb, nb), s);   // Lam(i, j) at XS[j nbp + i]
+  oz_slice_rows(P.XS.p, nbp, nb, nb, 1, P.oz_lamt.operand(nb, nb), s);   // its transpose
   const double* A = nullptr;
   const double* E = nullptr;
   if (kd > 0) {
@@ -585,6 +620,7 @@ void form_splus64(PatternData& P, cudaStream_t s) {
   const int nb = P.n_b, nbp = P.nbpad, kd = P.kdim;
   const size_t nn = (size_t)nb * nb;
   lauum(P.XS.p, nbp, nbp, nb, P.S64.p, nb, s);   // S^+ = X^T X
+  if (nb >= OZ_LOCAL_MIN_NB) oz_slice_rows(P.S64.p, nb, nb, nb, 0, P.oz_S.operand(), s);
   const double* Sdag = P.S64.p;
   if (kd > 0) {
     form_sdag64(P, s);
@@ -686,24 +722,18 @@ double factor_flops(const PatternData& P) {
   return f;
 }
 
-void check_tc_error(fetirp_ctx ctx);
-
 void factorize_patterns(fetirp_ctx ctx, const std::vector<PatternData*>& pats) {
   double flops = 0.0;
   for (const PatternData* P : pats) flops += factor_flops(*P);
   PhaseScope ph(ctx, FETIRP_PHASE_FACTOR, flops, 0.0);
   const size_t np = pats.size();
+  ensure_tc_error(ctx);
   fork_patterns(ctx, np);
   for (size_t i = 0; i < np; ++i) factor_stage_a(*pats[i], ctx->opt.pivot_tol, ctx->fstreams[i]);
   for (size_t i = 0; i < np; ++i) FETIRP_CUDA(cudaStreamSynchronize(ctx->fstreams[i]));
   for (size_t i = 0; i < np; ++i) {
     factor_check(*pats[i]);
     pats[i]->upload_zpiv(ctx->fstreams[i]);
-  }
-  if (!ctx->tc_error.p) {   // zeroed before the pattern streams run (they were forked earlier)
-    ctx->tc_error.alloc(1);
-    ctx->tc_error.zero(ctx->stream);
-    FETIRP_CUDA(cudaStreamSynchronize(ctx->stream));
   }
   for (size_t i = 0; i < np; ++i) factor_stage_b(*pats[i], ctx->tc_error.p, ctx->fstreams[i]);
   join_patterns(ctx, np);
@@ -776,6 +806,27 @@ void set_factored(LocalProblem& LP, int p, const PatternData& P, double* W) {
   LP.W[p] = W;
 }
 
+// Scratch slices of the right-hand sides of the sliced FP64 products: pattern p's tiles from tile_off[p], its exponents
+// from row_off[p].
+struct OzRhs {
+  long long tiles = 0, rows = 0;
+  long long tile_off[MAXP] = {}, row_off[MAXP] = {};
+  bool on[MAXP] = {};
+  void add(int p, int n_b, int n_rhs) {
+    on[p] = n_b >= OZ_LOCAL_MIN_NB && (long long)n_b * n_b * n_rhs >= OZ_LOCAL_MIN_FMAS;
+    tile_off[p] = tiles;
+    row_off[p] = rows;
+    if (!on[p]) return;
+    tiles += oz_tiles(n_rhs, n_b);
+    rows += round_up(n_rhs, 64);
+  }
+  void ensure(OzBuf& b) const {
+    b.slices.ensure((size_t)tiles * OZ_TILE);
+    b.exps.ensure((size_t)rows);
+  }
+  OzOperand at(const OzBuf& b, int p) const { return {b.slices.p + (size_t)tile_off[p] * OZ_TILE, b.exps.p + row_off[p]}; }
+};
+
 void ensure_apply_buffers(fetirp_ctx ctx, int k) {
   long long total = 0, total8 = 0;
   for (size_t p = 0; p < ctx->pats.size(); ++p) {
@@ -785,6 +836,10 @@ void ensure_apply_buffers(fetirp_ctx ctx, int k) {
   total = std::max(total, total8);   // the bf16 products use the FP32 buffers with leading dimension ld_y8
   ctx->Y64.ensure(total); ctx->Z64.ensure(total);
   if (factored_f64(ctx)) ctx->W64.ensure(total);
+  OzRhs R;
+  for (size_t p = 0; p < ctx->pats.size(); ++p)
+    R.add((int)p, ctx->pats[p]->n_b, (int)ctx->use[p].occs.size() * k);
+  R.ensure(ctx->oz_rhs);
   ctx->Y32.ensure(total); ctx->Z32.ensure(total); ctx->Ylo32.ensure(total);
   TcProblem T;   // would the tensor-core product split its reduction dimension?
   T.n_pat = (int)ctx->pats.size();
@@ -1232,7 +1287,7 @@ void build_structure(fetirp_ctx ctx, int64_t n_lambda, const double* c_host, con
   ctx->eta_part.ensure((size_t)(eta_chunks(nl) + ETA_GROUPS) * k * (k + 1)); ctx->T.ensure((size_t)k * k); ctx->alpha.ensure(k);
   ctx->n_kept.ensure(1);
   ctx->d_state.ensure(4);
-  if (!ctx->tc_error.p) { ctx->tc_error.alloc(1); ctx->tc_error.zero(s); }
+  ensure_tc_error(ctx);
   tc_init();
   ensure_apply_buffers(ctx, k);
   if (ctx->gc.exec) { cudaGraphExecDestroy(ctx->gc.exec); ctx->gc.exec = nullptr; }   // buffers may have moved
@@ -1273,6 +1328,56 @@ void project(fetirp_ctx ctx, double* V, int k) {
   g_apply(ctx->L, ctx->Ac.p, k, -1.0, 1.0, V, s);
 }
 
+// Z_p = S_p^+ Y_p in FP64: sliced products for the patterns large enough, FP64 FMAs for the others.  A pattern without
+// a formed S^+ (X[p]) goes through its factor, Lam^T (Lam Y), as two products.
+void local_f64(fetirp_ctx ctx, LocalProblem LP) {
+  cudaStream_t s = ctx->stream;
+  OzRhs R;
+  for (int p = 0; p < LP.n_pat; ++p) R.add(p, LP.n_b[p], LP.n_rhs[p]);
+  if (R.tiles == 0) {
+    local_gemm_f64(LP, s);
+    return;
+  }
+  R.ensure(ctx->oz_rhs);
+  ensure_tc_error(ctx);
+  OzGemm G1, G2;
+  OzSliceBatch B1, B2;
+  G1.error = G2.error = ctx->tc_error.p;
+  auto add = [](OzGemm& G, const OzOperand& A, const OzOperand& B, int nb, int nr, int mode, double* Z, long long ld) {
+    const int i = G.n++;
+    G.A[i] = A; G.B[i] = B;
+    G.M[i] = G.K[i] = nb; G.N[i] = nr; G.mode[i] = mode; G.Z[i] = Z; G.ldz[i] = ld;
+  };
+  bool simt = false;
+  for (int p = 0; p < LP.n_pat; ++p) {
+    if (!R.on[p]) {
+      simt = simt || LP.n_rhs[p] > 0;
+      continue;
+    }
+    const PatternData& P = *ctx->pats[p];
+    const OzOperand B = R.at(ctx->oz_rhs, p);
+    B1.add((const double*)LP.Y[p], LP.ld[p], LP.n_rhs[p], LP.n_b[p], 0, B);
+    if (LP.X[p]) add(G1, P.oz_lam.operand(), B, LP.n_b[p], LP.n_rhs[p], 1, LP.W[p], LP.ld[p]);
+    else add(G1, P.oz_S.operand(), B, LP.n_b[p], LP.n_rhs[p], 0, (double*)LP.Z[p], LP.ld[p]);
+  }
+  oz_slice(B1, s);
+  oz_gemm(G1, s);
+  for (int p = 0; p < LP.n_pat; ++p) {
+    if (!R.on[p]) continue;
+    if (LP.X[p]) {
+      const OzOperand B = R.at(ctx->oz_rhs, p);
+      B2.add(LP.W[p], LP.ld[p], LP.n_rhs[p], LP.n_b[p], 0, B);
+      add(G2, ctx->pats[p]->oz_lamt.operand(), B, LP.n_b[p], LP.n_rhs[p], 2, (double*)LP.Z[p], LP.ld[p]);
+    }
+    LP.n_rhs[p] = 0;
+  }
+  if (G2.n) {
+    oz_slice(B2, s);
+    oz_gemm(G2, s);
+  }
+  if (simt) local_gemm_f64(LP, s);
+}
+
 // gather -> local products -> scatter, each bracketed as its own phase
 template <typename T>
 void run_local(fetirp_ctx ctx, const Layout& L, const double* src, double* out, int k, const PatView<T>& Yv,
@@ -1292,7 +1397,7 @@ void run_local(fetirp_ctx ctx, const Layout& L, const double* src, double* out, 
   }
   {
     PhaseScope ph(ctx, FETIRP_PHASE_LOCAL, flops, sbytes + 2.0 * rhs_elems * es);
-    if (es == 8.0) local_gemm_f64(LP, s);
+    if (es == 8.0) local_f64(ctx, LP);
     else local_gemm_f32(LP, s);
   }
   {
@@ -1348,7 +1453,7 @@ void apply_F(fetirp_ctx ctx, const double* in, double* out, int k, int prec, boo
     run_local<float>(ctx, L, src, out, k, Yv, Zv, LP, 4.0);
   } else if (prec == FETIRP_PREC_TF32X3) {
     ctx->Y32.ensure(total); ctx->Ylo32.ensure(total); ctx->Z32.ensure(total);
-    if (!ctx->tc_error.p) { ctx->tc_error.alloc(1); ctx->tc_error.zero(s); }
+    ensure_tc_error(ctx);
     PatView<float> Yh{}, Yl{}, Zv{};
     TcProblem T;
     T.n_pat = n_pat;
@@ -1392,7 +1497,7 @@ void apply_F(fetirp_ctx ctx, const double* in, double* out, int k, int prec, boo
       total8 += (long long)ctx->use[p].occs.size() * k * ctx->pats[p]->ld_y8;
     }
     ctx->Y32.ensure(total8); ctx->Ylo32.ensure(total8); ctx->Z32.ensure(total8);
-    if (!ctx->tc_error.p) { ctx->tc_error.alloc(1); ctx->tc_error.zero(s); }
+    ensure_tc_error(ctx);
     PatView<__nv_bfloat16> Yh{}, Yl{};
     PatView<float> Zv{};
     TcProblem T;
@@ -3061,7 +3166,7 @@ void apply_split(fetirp_ctx ctx, const double* d_r, double* d_Q, int prec) {
       PairView<float> Yl{};
       view(SP.Ylo32.p, Yl);
       gather_pairs_split(L, SP.Vs.p, k, SP.d_pair_occ.p, SP.d_pair_g.p, SP.n_pairs, Y, Yl, s);
-      if (!ctx->tc_error.p) { ctx->tc_error.alloc(1); ctx->tc_error.zero(s); }
+      ensure_tc_error(ctx);
       TcProblem T;
       T.n_pat = n_pat;
       for (int p = 0; p < n_pat; ++p) {

@@ -38,14 +38,14 @@ struct Request {
 };
 
 // Device memory a structure will hold while it is solved: work blocks, direction history (capped by the slot
-// options), local traces and products, per-pattern loads and solutions.
+// options), local traces and products with the digit slices of FP64 right-hand sides, per-pattern loads and solutions.
 int64_t estimate_bytes(const Request& r, const fetirp_options& o) {
   const double nl = (double)r.n_lambda;
   const int k = r.k > 0 ? r.k : std::max(1, std::min(o.block_k, r.n_occ));
   const double ndofs = (double)r.f_offset.back();
   const double hist = o.history_bytes > 0 ? (double)o.history_bytes
                                           : 2.0 * 8.0 * nl * std::min<double>(nl, (double)o.max_iter * k);
-  const double work = 8.0 * nl * (12.0 + 6.0 * k) + 2.0 * 8.0 * ndofs + 5.0 * 8.0 * ndofs / 4.0 * k;
+  const double work = 8.0 * nl * (12.0 + 6.0 * k) + 2.0 * 8.0 * ndofs + 7.0 * 8.0 * ndofs / 4.0 * k;
   return (int64_t)(hist + work);
 }
 
