@@ -1301,8 +1301,14 @@ void build_structure(fetirp_ctx ctx, int64_t n_lambda, const double* c_host, con
 // ----------------------------------------------------------------------------------------- operators
 // V <- P V = V - G (G^T G)^{-1} G^T V (Eq. 6), FP64 throughout: with the rigid modes of elasticity G^T G is
 // ill-conditioned enough that FP32 products leave G-components that make the inner operator nonsymmetric.
-void project(fetirp_ctx ctx, double* V, int k) {
-  if (ctx->n_G == 0) return;
+void project(fetirp_ctx ctx, double* V, int k, const double* in = nullptr) {   // V <- P in (V by default)
+  if (!in) in = V;
+  if (ctx->n_G == 0) {
+    if (in != V)
+      FETIRP_CUDA(cudaMemcpyAsync(V, in, sizeof(double) * (size_t)ctx->L.n_lambda * k, cudaMemcpyDeviceToDevice,
+                                  ctx->stream));
+    return;
+  }
   cudaStream_t s = ctx->stream;
   const double nl = ctx->L.n_lambda, nG = ctx->n_G;
   // G^T V and G A: 2 flops per coefficient of G (sign N_b[j][m] per link) and column, each; (G^T G)^{-1} X
@@ -1316,6 +1322,8 @@ void project(fetirp_ctx ctx, double* V, int k) {
     float* ah = xl + (size_t)ctx->n_G * 64;
     float* al = ah + (size_t)ctx->n_G * 64;
     const long long ng2 = (long long)ctx->n_G * ctx->n_G;
+    if (in != V)
+      FETIRP_CUDA(cudaMemcpyAsync(V, in, sizeof(double) * (size_t)ctx->L.n_lambda * k, cudaMemcpyDeviceToDevice, s));
     gt_v_ds(ctx->L, V, k, ctx->Xc.p, s);
     split_pairs(ngk, ctx->Xc.p, xh, xl, s);
     small_gemm_ds(ctx->n_G, k, ctx->ds_ginv.p, ctx->ds_ginv.p + ng2, xh, xl, ctx->Ac.p, s, ctx->sg_part.p);
@@ -1323,9 +1331,9 @@ void project(fetirp_ctx ctx, double* V, int k) {
     g_apply_ds(ctx->L, ah, al, k, -1.0, 1.0, V, s);
     return;
   }
-  gt_v(ctx->L, V, k, ctx->Xc.p, s);
+  gt_v(ctx->L, in, k, ctx->Xc.p, s);
   small_gemm(ctx->n_G, k, ctx->Ginv.p, ctx->Xc.p, ctx->Ac.p, s, ctx->sg_part.p);
-  g_apply(ctx->L, ctx->Ac.p, k, -1.0, 1.0, V, s);
+  g_apply(ctx->L, ctx->Ac.p, k, -1.0, 1.0, V, s, in);
 }
 
 // Z_p = S_p^+ Y_p in FP64: sliced products for the patterns large enough, FP64 FMAs for the others.  A pattern without
@@ -1414,8 +1422,7 @@ void apply_F(fetirp_ctx ctx, const double* in, double* out, int k, int prec, boo
   const double* src = in;
   if (project_in && ctx->n_G > 0) {
     ctx->V2.ensure((size_t)L.n_lambda * k);
-    FETIRP_CUDA(cudaMemcpyAsync(ctx->V2.p, in, sizeof(double) * (size_t)L.n_lambda * k, cudaMemcpyDeviceToDevice, s));
-    project(ctx, ctx->V2.p, k);
+    project(ctx, ctx->V2.p, k, in);
     src = ctx->V2.p;
   }
   const int n_pat = (int)ctx->pats.size();

@@ -18,37 +18,44 @@ __device__ __forceinline__ double trace_of(const Layout& L, const double* __rest
 }
 
 // X[gofs(s)+m][g] = sum_{links (row, e) of s} (sign Nb[j])[m] * V[row][g], the signed coefficients taken from the
-// per-row tables.  Grid (occurrence, chunk of its links); warp w takes every 8th link of the chunk, four links
-// at a time (independent loads: link code, then its row of V and its coefficients), lane = column g (and g + 32
-// for k <= 64), so every link reads one contiguous row of V.  The warps' sums are added in warp order; with
+// per-row tables.  Grid (occurrence, chunk of its links).  KL lanes per link (k <= KL <= 32, a power of two; WIDE: two
+// columns per lane, k <= 64): a warp works on 32 / KL links at once, lane (sub, g) on column g, and takes four links
+// per step (independent loads: link code, then its row of V and its coefficients).  The kernel is bound by the FP64
+// pipe, which issues a warp's FMA at the same cost however many lanes hold a column: with a lane per column of 32, a
+// block of four columns took 290 us on 427,392 rows (192 occurrences); with 4 lanes per link 56 us (floor 37 us: 20M
+// FMAs at 1.7 per clock and SM).  The lanes of a column are added by shuffles, the warps' sums in warp order; with
 // several chunks per occurrence the last CTA of the occurrence (ticket) adds the chunks' partial sums in chunk
 // order and re-arms the ticket (deterministic, no atomics on values).
 constexpr int GTV_THREADS = 256;
 constexpr int MAX_KDIM = 6;
-template <bool WIDE>   // WIDE: 32 < k <= 64 (two columns per lane)
+template <int KL, bool WIDE>
 __global__ void __launch_bounds__(GTV_THREADS, WIDE ? 2 : 3) k_gt_v(Layout L, const double* __restrict__ V, int k,
                                                           double* __restrict__ X, int chunk) {
+  static_assert(!WIDE || KL == 32, "two columns per lane only with 32 lanes per link");
+  constexpr int SUB = 32 / KL;            // links a warp works on at once
+  constexpr int WORKERS = (GTV_THREADS / 32) * SUB;
   __shared__ double red[GTV_THREADS / 32][MAX_KDIM][64];
   __shared__ int s_last;
   const int s = blockIdx.x, c = blockIdx.y, nch = gridDim.y;
   const int kd = L.kdim[L.occ_pat[s]];
   const int l0 = L.slot_ptr[L.occ_obase[s]], nl = L.slot_ptr[L.occ_obase[s + 1]] - l0;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const bool c0 = lane < k, c1 = WIDE && lane + 32 < k;
+  const int g = lane % KL, sub = lane / KL, wid = w * SUB + sub;
+  const bool c0 = g < k, c1 = WIDE && g + 32 < k;
   const int i_end = min(nl, (c + 1) * chunk);
   double a0[MAX_KDIM] = {}, a1[MAX_KDIM] = {};
   if (kd > 0) {
-    for (int i = c * chunk + w; i < i_end; i += 32) {
+    for (int i = c * chunk + wid; i < i_end; i += 4 * WORKERS) {
       int code[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) code[u] = i + 8 * u < i_end ? L.slot_code[l0 + i + 8 * u] : -1;
+      for (int u = 0; u < 4; ++u) code[u] = i + WORKERS * u < i_end ? L.slot_code[l0 + i + WORKERS * u] : -1;
       double v0[4], v1[4], cf[4][MAX_KDIM];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int cu = max(code[u], 0);
-        const double* vr = V + (size_t)(cu >> 1) * k + lane;
-        v0[u] = c0 ? vr[0] : 0.0;
-        v1[u] = WIDE && c1 ? vr[32] : 0.0;
+        const double* vr = V + (size_t)(cu >> 1) * k + g;
+        v0[u] = c0 && code[u] >= 0 ? vr[0] : 0.0;   // no link: neither its row's value nor its coefficients
+        v1[u] = WIDE && c1 && code[u] >= 0 ? vr[32] : 0.0;
         const double* cp = L.rowg_coef + (size_t)cu * MAX_KDIM;
 #pragma unroll
         for (int m = 0; m < MAX_KDIM; ++m) cf[u][m] = (m < kd && code[u] >= 0) ? cp[m] : 0.0;
@@ -56,29 +63,36 @@ __global__ void __launch_bounds__(GTV_THREADS, WIDE ? 2 : 3) k_gt_v(Layout L, co
 #pragma unroll
       for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int m = 0; m < MAX_KDIM; ++m) {
-          a0[m] = fma(cf[u][m], v0[u], a0[m]);
-          if (WIDE) a1[m] = fma(cf[u][m], v1[u], a1[m]);
-        }
+        for (int m = 0; m < MAX_KDIM; ++m)
+          if (m < kd) {
+            a0[m] = fma(cf[u][m], v0[u], a0[m]);
+            if (WIDE) a1[m] = fma(cf[u][m], v1[u], a1[m]);
+          }
     }
   }
 #pragma unroll
   for (int m = 0; m < MAX_KDIM; ++m) {
-    red[w][m][lane] = a0[m];
-    red[w][m][lane + 32] = a1[m];
+    if (m < kd) {
+#pragma unroll
+      for (int off = KL; off < 32; off <<= 1) a0[m] += __shfl_xor_sync(0xffffffffu, a0[m], off);
+    }
+    if (sub == 0) {
+      red[w][m][g] = a0[m];
+      if (WIDE) red[w][m][g + 32] = a1[m];
+    }
   }
   __syncthreads();
   const int t = threadIdx.x;
   double* part = L.gtv_part + (size_t)s * nch * MAX_KDIM * 64;
   for (int i = t; i < kd * k; i += blockDim.x) {
-    const int m = i / k, g = i % k;
+    const int m = i / k, gg = i % k;
     double v = 0.0;
 #pragma unroll
-    for (int q = 0; q < GTV_THREADS / 32; ++q) v += red[q][m][g];
+    for (int q = 0; q < GTV_THREADS / 32; ++q) v += red[q][m][gg];
     if (nch == 1)
-      X[(size_t)(L.occ_gofs[s] + m) * k + g] = v;
+      X[(size_t)(L.occ_gofs[s] + m) * k + gg] = v;
     else
-      part[((size_t)c * MAX_KDIM + m) * 64 + g] = v;
+      part[((size_t)c * MAX_KDIM + m) * 64 + gg] = v;
   }
   if (nch == 1) return;
   __threadfence();
@@ -88,38 +102,52 @@ __global__ void __launch_bounds__(GTV_THREADS, WIDE ? 2 : 3) k_gt_v(Layout L, co
   if (!s_last) return;
   __threadfence();
   for (int i = t; i < kd * k; i += blockDim.x) {
-    const int m = i / k, g = i % k;
+    const int m = i / k, gg = i % k;
     double v = 0.0;
-    for (int q = 0; q < nch; ++q) v += __ldcg(part + ((size_t)q * MAX_KDIM + m) * 64 + g);
-    X[(size_t)(L.occ_gofs[s] + m) * k + g] = v;
+    for (int q = 0; q < nch; ++q) v += __ldcg(part + ((size_t)q * MAX_KDIM + m) * 64 + gg);
+    X[(size_t)(L.occ_gofs[s] + m) * k + gg] = v;
   }
   if (t == 0) L.gtv_ticket[s] = 0u;
 }
 
-// out[row][g] = beta*out + alpha * sum over the row's slots: (sign Nb[j]) . A[gofs(s)..][g], from the per-row
+// out[row][g] = beta*in + alpha * sum over the row's slots: (sign Nb[j]) . A[gofs(s)..][g], from the per-row
 // tables (coarse column, kernel dimension and signed coefficients of each slot), so that the only dependent
-// load is A's (small, cache-resident)
-__global__ void k_g_apply(Layout L, const double* __restrict__ A, int k, double alpha, double beta,
-                          double* __restrict__ out) {
+// load is A's (small, cache-resident).  C columns per thread (C = 4 when k is a multiple of 4: the row's tables and
+// coefficients are read once for four columns; bound by the 12 FMAs per element of the FP64 pipe: 57 -> 45 us for
+// 427,392 x 4).  in may be out.
+template <int C>
+__global__ void k_g_apply(Layout L, const double* __restrict__ A, int k, double alpha, double beta, const double* in,
+                          double* out) {
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (long long)L.n_lambda * k) return;
-  const int row = (int)(idx / k), g = (int)(idx % k);
-  double acc = 0.0;
+  const int kc = k / C;
+  if (idx >= (long long)L.n_lambda * kc) return;
+  const int row = (int)(idx / kc), g = (int)(idx % kc) * C;
+  double acc[C];
+#pragma unroll
+  for (int c = 0; c < C; ++c) acc[c] = 0.0;
 #pragma unroll
   for (int e = 0; e < 2; ++e) {
     const int g0 = L.rowg_gofs[2 * row + e];
     if (g0 < 0) continue;
     const int kd = L.rowg_kd[2 * row + e];
-    const double* c = L.rowg_coef + (size_t)(2 * row + e) * MAX_KDIM;
+    const double* cf = L.rowg_coef + (size_t)(2 * row + e) * MAX_KDIM;
     const double* a = A + (size_t)g0 * k + g;
-    double t = 0.0;
+    double t[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) t[c] = 0.0;
 #pragma unroll
     for (int m = 0; m < MAX_KDIM; ++m)
-      if (m < kd) t = fma(c[m], a[(size_t)m * k], t);
-    acc += t;
+      if (m < kd) {
+        const double f = cf[m];
+#pragma unroll
+        for (int c = 0; c < C; ++c) t[c] = fma(f, a[(size_t)m * k + c], t[c]);
+      }
+#pragma unroll
+    for (int c = 0; c < C; ++c) acc[c] = e == 0 ? t[c] : acc[c] + t[c];
   }
-  double* o = out + idx;
-  *o = (beta == 0.0 ? 0.0 : beta * *o) + alpha * acc;
+  const size_t o = (size_t)row * k + g;
+#pragma unroll
+  for (int c = 0; c < C; ++c) out[o + c] = (beta == 0.0 ? 0.0 : beta * in[o + c]) + alpha * acc[c];
 }
 
 // ---- double-single forms of G^T V and G A (the projections inside the inner solves of the mixed forms) -------
@@ -624,13 +652,33 @@ __global__ void k_scatter_pairs(Layout L, PairView<TI> Z, int k, const int* __re
 }
 
 // ------------------------------------------------------------------------------------------------ host
+// Chunk of links per CTA of G^T V: the layout's (sized for 32 lanes per link), or, when a warp works on several links at
+// once (k <= 16), long enough for about eight rounds of four links per worker, so that the loads in flight
+// rather than the per-CTA reduction and its ticket set the time; never more chunks than the layout's partials.
+struct GtvGrid { int chunk, chunks; };
+static GtvGrid gtv_grid(const Layout& L, int k) {
+  const int kl = k > 16 ? 32 : k > 8 ? 16 : k > 4 ? 8 : k > 1 ? 4 : 1;
+  const int workers = (GTV_THREADS / 32) * (32 / kl);
+  const int max_links = L.gtv_chunk * L.gtv_chunks;   // >= the links of the largest occurrence
+  int nch = L.gtv_chunks;
+  if (8 * 4 * workers > L.gtv_chunk) nch = std::max(1, std::min(nch, ceil_div(max_links, 8 * 4 * workers)));
+  // enough CTAs for the SMs come before the rounds per worker
+  nch = std::min(L.gtv_chunks, std::max(nch, ceil_div(2 * 152, std::max(L.n_occ, 1))));
+  const int chunk = (int)round_up(ceil_div(max_links, nch), 32);
+  return {chunk, ceil_div(max_links, chunk)};
+}
+
 void gt_v(const Layout& L, const double* V, int k, double* X, cudaStream_t s) {
   if (L.n_occ == 0) return;
   if (k > 64) throw Error(1, "k > 64");
-  if (k > 32)
-    k_gt_v<true><<<dim3(L.n_occ, L.gtv_chunks), GTV_THREADS, 0, s>>>(L, V, k, X, L.gtv_chunk);
-  else
-    k_gt_v<false><<<dim3(L.n_occ, L.gtv_chunks), GTV_THREADS, 0, s>>>(L, V, k, X, L.gtv_chunk);
+  const GtvGrid c = gtv_grid(L, k);
+  const dim3 grid(L.n_occ, c.chunks);
+  if (k > 32) k_gt_v<32, true><<<grid, GTV_THREADS, 0, s>>>(L, V, k, X, c.chunk);
+  else if (k > 16) k_gt_v<32, false><<<grid, GTV_THREADS, 0, s>>>(L, V, k, X, c.chunk);
+  else if (k > 8) k_gt_v<16, false><<<grid, GTV_THREADS, 0, s>>>(L, V, k, X, c.chunk);
+  else if (k > 4) k_gt_v<8, false><<<grid, GTV_THREADS, 0, s>>>(L, V, k, X, c.chunk);
+  else if (k > 1) k_gt_v<4, false><<<grid, GTV_THREADS, 0, s>>>(L, V, k, X, c.chunk);
+  else k_gt_v<1, false><<<grid, GTV_THREADS, 0, s>>>(L, V, k, X, c.chunk);
   FETIRP_LAUNCH_CHECK();
 }
 
@@ -639,16 +687,9 @@ void gt_v_ds(const Layout& L, const double* V, int k, double* X, cudaStream_t s)
   if (L.n_occ == 0) return;
   if (k > 64) throw Error(1, "k > 64");
   if (!L.rowg_coef_hi) throw Error(1, "double-single coefficients of G not built");
-  // Chunk of links per CTA: the layout's (sized for 32 lanes per link), or, when a warp works on several links at
-  // once (k <= 16), long enough for about eight rounds of four links per worker, so that the loads in flight
-  // rather than the per-CTA reduction and its ticket set the time; never more chunks than the layout's partials.
-  const int kl = k > 16 ? 32 : k > 8 ? 16 : k > 4 ? 8 : 4;
-  const int workers = (GTV_THREADS / 32) * (32 / kl);
-  const int max_links = L.gtv_chunk * L.gtv_chunks;   // >= the links of the largest occurrence
-  int nch = L.gtv_chunks;
-  if (8 * 4 * workers > L.gtv_chunk) nch = std::max(1, std::min(nch, ceil_div(max_links, 8 * 4 * workers)));
-  const int chunk = (int)round_up(ceil_div(max_links, nch), 32);
-  const dim3 grid(L.n_occ, ceil_div(max_links, chunk));
+  const GtvGrid c = gtv_grid(L, std::max(k, 2));
+  const int chunk = c.chunk;
+  const dim3 grid(L.n_occ, c.chunks);
   if (k > 32) k_gt_v_ds<32, true><<<grid, GTV_THREADS, 0, s>>>(L, V, k, X, chunk);
   else if (k > 16) k_gt_v_ds<32, false><<<grid, GTV_THREADS, 0, s>>>(L, V, k, X, chunk);
   else if (k > 8) k_gt_v_ds<16, false><<<grid, GTV_THREADS, 0, s>>>(L, V, k, X, chunk);
@@ -735,13 +776,15 @@ void g_apply_ds(const Layout& L, const float* Ah, const float* Al, int k, double
   FETIRP_LAUNCH_CHECK();
 }
 
-void g_apply(const Layout& L, const double* A, int k, double alpha, double beta, double* out, cudaStream_t s) {
-  long long n = (long long)L.n_lambda * k;
+void g_apply(const Layout& L, const double* A, int k, double alpha, double beta, double* out, cudaStream_t s,
+             const double* in) {
+  const long long n = (long long)L.n_lambda * k;
   if (n == 0) return;
-  k_g_apply<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(L, A, k, alpha, beta, out);
+  if (!in) in = out;
+  if (k % 4 == 0) k_g_apply<4><<<(unsigned)((n / 4 + 255) / 256), 256, 0, s>>>(L, A, k, alpha, beta, in, out);
+  else k_g_apply<1><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(L, A, k, alpha, beta, in, out);
   FETIRP_LAUNCH_CHECK();
 }
-
 
 void gtg_dense(const Layout& L, const int*, const int*, int n_pairs, const int* pair_s, const int* pair_t,
                double* GtG, cudaStream_t s) {

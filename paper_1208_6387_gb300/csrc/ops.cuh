@@ -76,7 +76,8 @@ struct Layout {
 // X[gofs(s) + m][g] = sum over links (row, sign) of s: sign * Nb[j][m] * V[row][g]   (X = G^T V)
 void gt_v(const Layout& L, const double* V, int k, double* X, cudaStream_t s);
 // out[row][g] = beta * out[row][g] + alpha * (G A)[row][g]
-void g_apply(const Layout& L, const double* A, int k, double alpha, double beta, double* out, cudaStream_t s);
+void g_apply(const Layout& L, const double* A, int k, double alpha, double beta, double* out, cudaStream_t s,
+             const double* in = nullptr);   // beta in + alpha G A (in: out by default)
 // Double-single forms (FP32 pairs, ~2^-46 relative; the inner solves of the mixed forms): X = G^T V, and
 // out = beta out + alpha G A with A given as pairs Ah + Al (split_pairs); need Layout.rowg_coef_hi/lo.
 void gt_v_ds(const Layout& L, const double* V, int k, double* X, cudaStream_t s);

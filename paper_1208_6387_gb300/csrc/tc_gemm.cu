@@ -244,14 +244,25 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS));
 }
 
-// Z = sum of the K-split partials in split order (the first n_b rows of every column), one thread per element
-__global__ void k_tc_reduce(const float* __restrict__ part, int splits, long long count, int n_b, long long ld,
-                            float* __restrict__ Z) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= count || (int)(i % ld) >= n_b) return;
+// Z = sum of the K-split partials in split order (the first n_b rows of every column), one thread per element; blocks
+// blk_off[p] .. of pattern p
+struct TcReduce {
+  const float* part[TC_MAXP];
+  float* Z[TC_MAXP];
+  long long count[TC_MAXP], ld[TC_MAXP];
+  int n_b[TC_MAXP], blk_off[TC_MAXP];
+  int n, splits;
+};
+__global__ void k_tc_reduce(const __grid_constant__ TcReduce R) {
+  int p = 0;
+  while (p + 1 < R.n && (int)blockIdx.x >= R.blk_off[p + 1]) ++p;
+  const long long i = (long long)((int)blockIdx.x - R.blk_off[p]) * blockDim.x + threadIdx.x;
+  const long long count = R.count[p];
+  if (i >= count || (int)(i % R.ld[p]) >= R.n_b[p]) return;
+  const float* part = R.part[p];
   float acc = part[i];
-  for (int q = 1; q < splits; ++q) acc += part[(size_t)q * count + i];
-  Z[i] = acc;
+  for (int q = 1; q < R.splits; ++q) acc += part[(size_t)q * count + i];
+  R.Z[p][i] = acc;
 }
 
 __global__ void k_split_tf32(const double* __restrict__ x, long long rows, long long cols, long long ld_in,
@@ -417,13 +428,20 @@ void tc_gemm_split(const TcProblem& T, bool bf16, int* d_error, cudaStream_t s) 
     if (bf16) k_tc_gemm<true><<<total * splits, THREADS, SMEM_BYTES, s>>>(P);
     else k_tc_gemm<false><<<total * splits, THREADS, SMEM_BYTES, s>>>(P);
     FETIRP_LAUNCH_CHECK();
-    if (splits > 1)
+    if (splits > 1) {
+      TcReduce R;
+      R.n = P.n_pat;
+      R.splits = splits;
+      int blocks = 0;
       for (int i = 0; i < P.n_pat; ++i) {
-        const long long count = (long long)P.n_rhs[i] * P.ldz[i];
-        k_tc_reduce<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(P.part[i], splits, count, P.n_b[i], P.ldz[i],
-                                                                    P.Z[i]);
-        FETIRP_LAUNCH_CHECK();
+        R.part[i] = P.part[i]; R.Z[i] = P.Z[i]; R.ld[i] = P.ldz[i]; R.n_b[i] = P.n_b[i];
+        R.count[i] = (long long)P.n_rhs[i] * P.ldz[i];
+        R.blk_off[i] = blocks;
+        blocks += ceil_div(R.count[i], 256);
       }
+      k_tc_reduce<<<blocks, 256, 0, s>>>(R);
+      FETIRP_LAUNCH_CHECK();
+    }
   }
 }
 }  // namespace
