@@ -18,43 +18,42 @@ __device__ __forceinline__ double trace_of(const Layout& L, const double* __rest
 }
 
 // X[gofs(s)+m][g] = sum_{links (row, e) of s} (sign Nb[j])[m] * V[row][g], the signed coefficients taken from the
-// per-row tables.  Grid (occurrence, chunk of its links).  KL lanes per link (k <= KL <= 32, a power of two; WIDE: two
-// columns per lane, k <= 64): a warp works on 32 / KL links at once, lane (sub, g) on column g, and takes four links
-// per step (independent loads: link code, then its row of V and its coefficients).  The kernel is bound by the FP64
-// pipe, which issues a warp's FMA at the same cost however many lanes hold a column: with a lane per column of 32, a
-// block of four columns took 290 us on 427,392 rows (192 occurrences); with 4 lanes per link 56 us (floor 37 us: 20M
-// FMAs at 1.7 per clock and SM).  The lanes of a column are added by shuffles, the warps' sums in warp order; with
-// several chunks per occurrence the last CTA of the occurrence (ticket) adds the chunks' partial sums in chunk
-// order and re-arms the ticket (deterministic, no atomics on values).
+// per-row tables.  An occurrence's links are cut into chunks, a chunk over 8 workers: worker w takes every 8th link, four
+// at a time (independent loads: link code, then its row of V and its coefficients), the workers' sums are added in
+// order, then the chunks' (by the occurrence's last CTA, found by a ticket that it re-arms): deterministic, and the same
+// sum for every KL.  A worker is KL lanes, one per column (k <= KL; KL = 32 also k <= 64 with two columns per lane,
+// WIDE), so a CTA of 256 threads works on 32 / KL chunks.  The kernel is bound by the FP64 pipe, which charges a whole
+// warp for an FMA however many lanes hold a column: with 32 lanes per link a block of four columns took 290 us on
+// 427,392 rows (192 occurrences), with 4 lanes 66 us (floor 37 us: 20M FMAs at 1.7 per clock and SM).
 constexpr int GTV_THREADS = 256;
 constexpr int MAX_KDIM = 6;
 template <int KL, bool WIDE>
 __global__ void __launch_bounds__(GTV_THREADS, WIDE ? 2 : 3) k_gt_v(Layout L, const double* __restrict__ V, int k,
-                                                          double* __restrict__ X, int chunk) {
+                                                          double* __restrict__ X, int chunk, int nch) {
   static_assert(!WIDE || KL == 32, "two columns per lane only with 32 lanes per link");
-  constexpr int SUB = 32 / KL;            // links a warp works on at once
-  constexpr int WORKERS = (GTV_THREADS / 32) * SUB;
-  __shared__ double red[GTV_THREADS / 32][MAX_KDIM][64];
+  constexpr int CPC = 32 / KL;                      // chunks per CTA
+  constexpr int COLS = WIDE ? 64 : KL;
+  __shared__ double red[CPC][8][MAX_KDIM][COLS];
   __shared__ int s_last;
-  const int s = blockIdx.x, c = blockIdx.y, nch = gridDim.y;
+  const int s = blockIdx.x;
   const int kd = L.kdim[L.occ_pat[s]];
   const int l0 = L.slot_ptr[L.occ_obase[s]], nl = L.slot_ptr[L.occ_obase[s + 1]] - l0;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int g = lane % KL, sub = lane / KL, wid = w * SUB + sub;
+  const int g = threadIdx.x % KL, grp = threadIdx.x / KL, w = grp & 7, cl = grp >> 3;
+  const int c = blockIdx.y * CPC + cl;
   const bool c0 = g < k, c1 = WIDE && g + 32 < k;
-  const int i_end = min(nl, (c + 1) * chunk);
+  const int i_end = c < nch ? min(nl, (c + 1) * chunk) : 0;
   double a0[MAX_KDIM] = {}, a1[MAX_KDIM] = {};
   if (kd > 0) {
-    for (int i = c * chunk + wid; i < i_end; i += 4 * WORKERS) {
+    for (int i = c * chunk + w; i < i_end; i += 32) {
       int code[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) code[u] = i + WORKERS * u < i_end ? L.slot_code[l0 + i + WORKERS * u] : -1;
+      for (int u = 0; u < 4; ++u) code[u] = i + 8 * u < i_end ? L.slot_code[l0 + i + 8 * u] : -1;
       double v0[4], v1[4], cf[4][MAX_KDIM];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int cu = max(code[u], 0);
         const double* vr = V + (size_t)(cu >> 1) * k + g;
-        v0[u] = c0 && code[u] >= 0 ? vr[0] : 0.0;   // no link: neither its row's value nor its coefficients
+        v0[u] = c0 && code[u] >= 0 ? vr[0] : 0.0;   // no link: neither a row's value nor its coefficients
         v1[u] = WIDE && c1 && code[u] >= 0 ? vr[32] : 0.0;
         const double* cp = L.rowg_coef + (size_t)cu * MAX_KDIM;
 #pragma unroll
@@ -72,42 +71,41 @@ __global__ void __launch_bounds__(GTV_THREADS, WIDE ? 2 : 3) k_gt_v(Layout L, co
   }
 #pragma unroll
   for (int m = 0; m < MAX_KDIM; ++m) {
-    if (m < kd) {
-#pragma unroll
-      for (int off = KL; off < 32; off <<= 1) a0[m] += __shfl_xor_sync(0xffffffffu, a0[m], off);
-    }
-    if (sub == 0) {
-      red[w][m][g] = a0[m];
-      if (WIDE) red[w][m][g + 32] = a1[m];
-    }
+    red[cl][w][m][g] = a0[m];
+    if (WIDE) red[cl][w][m][g + 32] = a1[m];
   }
   __syncthreads();
   const int t = threadIdx.x;
   double* part = L.gtv_part + (size_t)s * nch * MAX_KDIM * 64;
-  for (int i = t; i < kd * k; i += blockDim.x) {
-    const int m = i / k, gg = i % k;
+  const int nc = min(CPC, nch - (int)blockIdx.y * CPC);
+  for (int i = t; i < nc * kd * k; i += blockDim.x) {
+    const int q0 = i / (kd * k), m = i / k % kd, gg = i % k;
     double v = 0.0;
 #pragma unroll
-    for (int q = 0; q < GTV_THREADS / 32; ++q) v += red[q][m][gg];
+    for (int q = 0; q < 8; ++q) v += red[q0][q][m][gg];
     if (nch == 1)
       X[(size_t)(L.occ_gofs[s] + m) * k + gg] = v;
     else
-      part[((size_t)c * MAX_KDIM + m) * 64 + gg] = v;
+      part[((size_t)(blockIdx.y * CPC + q0) * MAX_KDIM + m) * 64 + gg] = v;
   }
   if (nch == 1) return;
-  __threadfence();
-  __syncthreads();
-  if (t == 0) s_last = atomicAdd(&L.gtv_ticket[s], 1u) == (unsigned)(nch - 1);
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
+  if (gridDim.y > 1) {
+    __threadfence();
+    __syncthreads();
+    if (t == 0) s_last = atomicAdd(&L.gtv_ticket[s], 1u) == gridDim.y - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+  } else {
+    __syncthreads();
+  }
   for (int i = t; i < kd * k; i += blockDim.x) {
     const int m = i / k, gg = i % k;
     double v = 0.0;
     for (int q = 0; q < nch; ++q) v += __ldcg(part + ((size_t)q * MAX_KDIM + m) * 64 + gg);
     X[(size_t)(L.occ_gofs[s] + m) * k + gg] = v;
   }
-  if (t == 0) L.gtv_ticket[s] = 0u;
+  if (t == 0 && gridDim.y > 1) L.gtv_ticket[s] = 0u;
 }
 
 // out[row][g] = beta*in + alpha * sum over the row's slots: (sign Nb[j]) . A[gofs(s)..][g], from the per-row
@@ -652,33 +650,16 @@ __global__ void k_scatter_pairs(Layout L, PairView<TI> Z, int k, const int* __re
 }
 
 // ------------------------------------------------------------------------------------------------ host
-// Chunk of links per CTA of G^T V: the layout's (sized for 32 lanes per link), or, when a warp works on several links at
-// once (k <= 16), long enough for about eight rounds of four links per worker, so that the loads in flight
-// rather than the per-CTA reduction and its ticket set the time; never more chunks than the layout's partials.
-struct GtvGrid { int chunk, chunks; };
-static GtvGrid gtv_grid(const Layout& L, int k) {
-  const int kl = k > 16 ? 32 : k > 8 ? 16 : k > 4 ? 8 : k > 1 ? 4 : 1;
-  const int workers = (GTV_THREADS / 32) * (32 / kl);
-  const int max_links = L.gtv_chunk * L.gtv_chunks;   // >= the links of the largest occurrence
-  int nch = L.gtv_chunks;
-  if (8 * 4 * workers > L.gtv_chunk) nch = std::max(1, std::min(nch, ceil_div(max_links, 8 * 4 * workers)));
-  // enough CTAs for the SMs come before the rounds per worker
-  nch = std::min(L.gtv_chunks, std::max(nch, ceil_div(2 * 152, std::max(L.n_occ, 1))));
-  const int chunk = (int)round_up(ceil_div(max_links, nch), 32);
-  return {chunk, ceil_div(max_links, chunk)};
-}
-
 void gt_v(const Layout& L, const double* V, int k, double* X, cudaStream_t s) {
   if (L.n_occ == 0) return;
   if (k > 64) throw Error(1, "k > 64");
-  const GtvGrid c = gtv_grid(L, k);
-  const dim3 grid(L.n_occ, c.chunks);
-  if (k > 32) k_gt_v<32, true><<<grid, GTV_THREADS, 0, s>>>(L, V, k, X, c.chunk);
-  else if (k > 16) k_gt_v<32, false><<<grid, GTV_THREADS, 0, s>>>(L, V, k, X, c.chunk);
-  else if (k > 8) k_gt_v<16, false><<<grid, GTV_THREADS, 0, s>>>(L, V, k, X, c.chunk);
-  else if (k > 4) k_gt_v<8, false><<<grid, GTV_THREADS, 0, s>>>(L, V, k, X, c.chunk);
-  else if (k > 1) k_gt_v<4, false><<<grid, GTV_THREADS, 0, s>>>(L, V, k, X, c.chunk);
-  else k_gt_v<1, false><<<grid, GTV_THREADS, 0, s>>>(L, V, k, X, c.chunk);
+  const int chunk = L.gtv_chunk, nch = L.gtv_chunks;
+  auto grid = [&](int kl) { return dim3(L.n_occ, ceil_div(nch, 32 / kl)); };
+  if (k > 32) k_gt_v<32, true><<<grid(32), GTV_THREADS, 0, s>>>(L, V, k, X, chunk, nch);
+  else if (k > 16) k_gt_v<32, false><<<grid(32), GTV_THREADS, 0, s>>>(L, V, k, X, chunk, nch);
+  else if (k > 8) k_gt_v<16, false><<<grid(16), GTV_THREADS, 0, s>>>(L, V, k, X, chunk, nch);
+  else if (k > 4) k_gt_v<8, false><<<grid(8), GTV_THREADS, 0, s>>>(L, V, k, X, chunk, nch);
+  else k_gt_v<4, false><<<grid(4), GTV_THREADS, 0, s>>>(L, V, k, X, chunk, nch);
   FETIRP_LAUNCH_CHECK();
 }
 
@@ -687,9 +668,16 @@ void gt_v_ds(const Layout& L, const double* V, int k, double* X, cudaStream_t s)
   if (L.n_occ == 0) return;
   if (k > 64) throw Error(1, "k > 64");
   if (!L.rowg_coef_hi) throw Error(1, "double-single coefficients of G not built");
-  const GtvGrid c = gtv_grid(L, std::max(k, 2));
-  const int chunk = c.chunk;
-  const dim3 grid(L.n_occ, c.chunks);
+  // Chunk of links per CTA: the layout's (sized for 32 lanes per link), or, when a warp works on several links at
+  // once (k <= 16), long enough for about eight rounds of four links per worker, so that the loads in flight
+  // rather than the per-CTA reduction and its ticket set the time; never more chunks than the layout's partials.
+  const int kl = k > 16 ? 32 : k > 8 ? 16 : k > 4 ? 8 : 4;
+  const int workers = (GTV_THREADS / 32) * (32 / kl);
+  const int max_links = L.gtv_chunk * L.gtv_chunks;   // >= the links of the largest occurrence
+  int nch = L.gtv_chunks;
+  if (8 * 4 * workers > L.gtv_chunk) nch = std::max(1, std::min(nch, ceil_div(max_links, 8 * 4 * workers)));
+  const int chunk = (int)round_up(ceil_div(max_links, nch), 32);
+  const dim3 grid(L.n_occ, ceil_div(max_links, chunk));
   if (k > 32) k_gt_v_ds<32, true><<<grid, GTV_THREADS, 0, s>>>(L, V, k, X, chunk);
   else if (k > 16) k_gt_v_ds<32, false><<<grid, GTV_THREADS, 0, s>>>(L, V, k, X, chunk);
   else if (k > 8) k_gt_v_ds<16, false><<<grid, GTV_THREADS, 0, s>>>(L, V, k, X, chunk);

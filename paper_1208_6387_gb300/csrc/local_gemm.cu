@@ -43,14 +43,18 @@ __global__ void __launch_bounds__(256) k_local_gemm(LocalTiles LT) {
   const int kbeg = mode == 2 ? m0 / BK * BK : 0;
   const int kend = mode == 1 ? min(nb, m0 + BM) : nb;
   T acc[TM][TN] = {};
-  for (int k0 = kbeg; k0 < kend; k0 += BK) {
+  // The next K step is loaded into registers while the current one is multiplied: a small product runs one CTA per SM
+  // or less, and would otherwise wait out a load in every step (two patterns of n_b 888, 75 right-hand sides each, FP32:
+  // 28 -> 17 us).
+  T ra[LA], rb[LB];
+  auto fetch = [&](int k0) {
     if (mode == 1) {   // transposed storage: consecutive threads along i
 #pragma unroll
       for (int u = 0; u < LA; ++u) {
         const int idx = tid + 256 * u;
         const int r = idx % BM, kk = idx / BM;
         const int i = m0 + r, j = k0 + kk;
-        if (idx < BK * BM) sa[kk][r] = (i < nb && j <= i) ? A[(size_t)j * lda + i] : T(0);
+        ra[u] = (idx < BK * BM && i < nb && j <= i) ? A[(size_t)j * lda + i] : T(0);
       }
     } else {
 #pragma unroll
@@ -58,7 +62,7 @@ __global__ void __launch_bounds__(256) k_local_gemm(LocalTiles LT) {
         const int idx = tid + 256 * u;
         const int kk = idx % BK, r = idx / BK;
         const int i = m0 + r, j = k0 + kk;
-        if (idx < BK * BM) sa[kk][r] = (i < nb && j < nb && (mode == 0 || j >= i)) ? A[(size_t)i * lda + j] : T(0);
+        ra[u] = (idx < BK * BM && i < nb && j < nb && (mode == 0 || j >= i)) ? A[(size_t)i * lda + j] : T(0);
       }
     }
 #pragma unroll
@@ -66,9 +70,26 @@ __global__ void __launch_bounds__(256) k_local_gemm(LocalTiles LT) {
       const int idx = tid + 256 * u;
       const int kk = idx % BK, r = idx / BK;
       const int c = n0 + r, j = k0 + kk;
-      if (idx < BK * BN) sb[kk][r] = (c < nr && j < nb) ? Y[(long long)c * ld + j] : T(0);
+      rb[u] = (idx < BK * BN && c < nr && j < nb) ? Y[(long long)c * ld + j] : T(0);
+    }
+  };
+  if (kbeg < kend) fetch(kbeg);
+  for (int k0 = kbeg; k0 < kend; k0 += BK) {
+#pragma unroll
+    for (int u = 0; u < LA; ++u) {
+      const int idx = tid + 256 * u;
+      if (idx < BK * BM) {
+        if (mode == 1) sa[idx / BM][idx % BM] = ra[u];
+        else sa[idx % BK][idx / BK] = ra[u];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < LB; ++u) {
+      const int idx = tid + 256 * u;
+      if (idx < BK * BN) sb[idx % BK][idx / BK] = rb[u];
     }
     __syncthreads();
+    if (k0 + BK < kend) fetch(k0 + BK);
 #pragma unroll 16
     for (int kk = 0; kk < BK; ++kk) {
       T av[TM], bv[TN];

@@ -8,10 +8,12 @@
 // local products); bf16 pairs carry 16 (near 2^-16, at twice the tensor rate of tf32).  The FP64 outer
 // refinement of the solver removes either error.
 //
-// One CTA computes a 256 (rows of S^+) x 256 (right-hand sides) tile of one pattern as two 128 x 256 halves,
-// each an MMA of M = 128, N = 256 into its own TMEM accumulator (the two fill the 512 TMEM columns): both halves
-// use the same staged right-hand-side tile, so a K step loads 64 KB for 12 MMAs instead of 96 KB for 12 with one
-// 128-row half (operand bytes per flop from L2 are what limits this kernel).  Warp roles: warp 0 lane 0 issues
+// One CTA computes a bm (rows of S^+: 256 or 128) x bn (right-hand sides: 32 .. 256) tile of one pattern as one or two
+// 128 x bn halves, each an MMA of M = 128, N = bn into its own TMEM accumulator: both halves use the same staged
+// right-hand-side tile, so a 256 x 256 tile's K step loads 64 KB for 12 MMAs instead of 96 KB for 12 with one
+// 128-row half (operand bytes per flop from L2 are what limits this kernel).  The tile is chosen per launch (tc_tile):
+// smaller where large ones would leave SMs idle or mostly multiply padding.  Every output is the same sum in the
+// same order in any tile, bit for bit.  Warp roles: warp 0 lane 0 issues
 // TMA loads, warp 1 lane 0 issues the MMAs, all eight warps drain TMEM in the epilogue (warps w and w + 4 the
 // same 32 TMEM lanes of the two halves).  Every wait on an mbarrier is bounded: on expiry the CTA records an
 // error code, stops issuing work, waits (again bounded) for its own MMAs to retire, frees TMEM and returns.
@@ -29,17 +31,14 @@ namespace fetirp {
 
 namespace {
 
-// 256 x 256 output tile per CTA (two 128 x 256 halves)
-constexpr int BM = 256, BMH = 128, BN = 256;
+constexpr int BM = 256, BMH = 128, BN = 256;       // largest output tile of a CTA (two 128 x 256 halves)
 constexpr int ROW_BYTES = 64;                     // one K step of a tile row = one 64-byte swizzle row
-constexpr int STAGES = 3;
-constexpr int TILE_A_BYTES = BM * ROW_BYTES;      // 16 KB (both halves; the second starts 8 KB in)
-constexpr int TILE_B_BYTES = BN * ROW_BYTES;      // 16 KB
-constexpr int STAGE_BYTES = 2 * TILE_A_BYTES + 2 * TILE_B_BYTES;   // A_hi, A_lo, B_hi, B_lo: 64 KB
+constexpr int MAX_STAGES = 8;
+constexpr int RING_BYTES = 3 * 2 * (BM + BN) * ROW_BYTES;   // A_hi, A_lo, B_hi, B_lo per stage: 3 of 64 KB, or more smaller
 constexpr int TMEM_COLS = 2 * BN;                 // two FP32 accumulators of 256 columns
 constexpr int THREADS = 256;
 // stages, 1024 bytes of alignment slack, barriers and flags, and 4 KB of margin past the last stage
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256 + 4096;
+constexpr int SMEM_BYTES = RING_BYTES + 1024 + 256 + 4096;
 
 // Shared-memory matrix descriptor (tcgen05): K-major, 64-byte swizzle, 8-row groups 512 bytes apart.
 __device__ __forceinline__ uint64_t smem_desc(const void* p) {
@@ -53,14 +52,14 @@ __device__ __forceinline__ uint64_t smem_desc(const void* p) {
   return d;
 }
 
-// Instruction descriptor: D f32, A/B tf32 (kind::tf32) or bf16 (kind::f16), both K-major, N = BN, M = BM.
+// Instruction descriptor: D f32, A/B tf32 (kind::tf32) or bf16 (kind::f16), both K-major, N = bn, M = 128.
 template <bool BF16>
-__device__ __forceinline__ uint32_t instr_desc() {
+__device__ __forceinline__ uint32_t instr_desc(int bn) {
   uint32_t d = 0;
   d |= 1u << 4;                          // D format f32
   d |= (BF16 ? 1u : 2u) << 7;            // A format: bf16 (kind::f16) or tf32
   d |= (BF16 ? 1u : 2u) << 10;           // B format
-  d |= (uint32_t)(BN >> 3) << 17;   // N / 8
+  d |= (uint32_t)(bn >> 3) << 17;   // N / 8
   d |= (uint32_t)(BMH >> 4) << 24;  // M / 16 (one half)
   return d;
 }
@@ -69,11 +68,10 @@ struct TcParams {
   CUtensorMap a_hi[TC_MAXP], a_lo[TC_MAXP], b_hi[TC_MAXP], b_lo[TC_MAXP];
   float* Z[TC_MAXP];
   float* part[TC_MAXP];   // K-split partials of pattern p (splits copies of the Z layout), when splits > 1
-  int splits;
+  int splits, bm, bn, stages;
   long long ldz[TC_MAXP];
   int n_b[TC_MAXP];
   int n_rhs[TC_MAXP];
-  int tiles_m[TC_MAXP];
   int tile_off[TC_MAXP + 1];
   int n_pat;
   int* error;   // device flag: first failing CTA writes its code
@@ -88,9 +86,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
   constexpr int BK = ROW_BYTES / (BF16 ? 2 : 4);   // K elements per stage
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
-  uint64_t* empty = full + STAGES;
-  uint64_t* done = empty + STAGES;
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + RING_BYTES);
+  uint64_t* empty = full + MAX_STAGES;
+  uint64_t* done = empty + MAX_STAGES;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   volatile int* n_loaded = abort_flag + 1;     // stages whose TMA loads were issued
@@ -103,15 +101,17 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
   // right-hand-side tiles inner: the CTAs of a wave share few 128-row tiles of S (read from DRAM once, then
   // served from L2 to the other CTAs of the row), and Y (a few tens of MB per pattern) stays in L2
   const int t = tile - P.tile_off[p];
-  const int tiles_n = (P.n_rhs[p] + BN - 1) / BN;
-  const int m0 = (t / tiles_n) * BM, n0 = (t % tiles_n) * BN;
+  const int bm = P.bm, bn = P.bn, stages = P.stages;
+  const int a_bytes = bm * ROW_BYTES, b_bytes = bn * ROW_BYTES, stage_bytes = 2 * (a_bytes + b_bytes);
+  const int tiles_n = (P.n_rhs[p] + bn - 1) / bn;
+  const int m0 = (t / tiles_n) * bm, n0 = (t % tiles_n) * bn;
   const int nk_all = (P.n_b[p] + BK - 1) / BK;
   const int kb0 = (int)((long long)sp * nk_all / P.splits), kb1 = (int)((long long)(sp + 1) * nk_all / P.splits);
   const int nk = kb1 - kb0;   // K steps of this CTA
-  const bool two = m0 + BMH < P.n_b[p];   // the second 128-row half has rows of S (else its MMAs are skipped)
+  const bool two = bm > BMH && m0 + BMH < P.n_b[p];   // the second 128-row half has rows of S (else its MMAs are skipped)
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
+    for (int s = 0; s < stages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
@@ -134,30 +134,30 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
   if (warp == 0 && lane == 0) {
     // producer
     for (int kb = 0; kb < nk; ++kb) {
-      const int s = kb % STAGES;
-      const uint32_t ph = (kb / STAGES) & 1;
-      if (kb >= STAGES && !mbar_wait(&empty[s], ph ^ 1)) {
+      const int s = kb % stages;
+      const uint32_t ph = (kb / stages) & 1;
+      if (kb >= stages && !mbar_wait(&empty[s], ph ^ 1)) {
         atomicCAS(P.error, 0, 1);
         *abort_flag = 1;
         break;
       }
       if (*abort_flag) break;
-      uint8_t* st = smem + s * STAGE_BYTES;
-      mbar_expect_tx(&full[s], STAGE_BYTES);
+      uint8_t* st = smem + s * stage_bytes;
+      mbar_expect_tx(&full[s], stage_bytes);
       const int kx = (kb0 + kb) * BK;
       tma_load_2d(&P.a_hi[p], &full[s], st, kx, m0);
-      tma_load_2d(&P.a_lo[p], &full[s], st + TILE_A_BYTES, kx, m0);
-      tma_load_2d(&P.b_hi[p], &full[s], st + 2 * TILE_A_BYTES, kx, n0);
-      tma_load_2d(&P.b_lo[p], &full[s], st + 2 * TILE_A_BYTES + TILE_B_BYTES, kx, n0);
+      tma_load_2d(&P.a_lo[p], &full[s], st + a_bytes, kx, m0);
+      tma_load_2d(&P.b_hi[p], &full[s], st + 2 * a_bytes, kx, n0);
+      tma_load_2d(&P.b_lo[p], &full[s], st + 2 * a_bytes + b_bytes, kx, n0);
       *n_loaded = kb + 1;
     }
   } else if (warp == 1 && lane == 0) {
     // MMA issuer
-    const uint32_t idesc = instr_desc<BF16>();
+    const uint32_t idesc = instr_desc<BF16>(bn);
     int issued = 0;
     for (int kb = 0; kb < nk; ++kb) {
-      const int s = kb % STAGES;
-      const uint32_t ph = (kb / STAGES) & 1;
+      const int s = kb % stages;
+      const uint32_t ph = (kb / stages) & 1;
       if (!mbar_wait(&full[s], ph)) {
         atomicCAS(P.error, 0, 2);
         *abort_flag = 1;
@@ -166,14 +166,14 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
       *n_consumed = kb + 1;
       if (*abort_flag) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      uint8_t* st = smem + s * STAGE_BYTES;
-      const uint64_t bhi = smem_desc(st + 2 * TILE_A_BYTES), blo = smem_desc(st + 2 * TILE_A_BYTES + TILE_B_BYTES);
+      uint8_t* st = smem + s * stage_bytes;
+      const uint64_t bhi = smem_desc(st + 2 * a_bytes), blo = smem_desc(st + 2 * a_bytes + b_bytes);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         if (h == 1 && !two) break;
         // half h: rows h * 128 .. of the A tiles (8 KB in), accumulator at TMEM column h * BN
         const uint64_t ahi = smem_desc(st + h * (BMH * ROW_BYTES));
-        const uint64_t alo = smem_desc(st + TILE_A_BYTES + h * (BMH * ROW_BYTES));
+        const uint64_t alo = smem_desc(st + a_bytes + h * (BMH * ROW_BYTES));
         const uint32_t acc = tmem + (uint32_t)(h * BN);
 #pragma unroll
         for (int kk = 0; kk < ROW_BYTES / 32; ++kk) {
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
     const long long ldz = P.ldz[p];
     const int nr = P.n_rhs[p];
 #pragma unroll 1
-    for (int c0 = 0; c0 < BN; c0 += 32) {
+    for (int c0 = 0; c0 < bn; c0 += 32) {
       uint32_t v[32];
       const uint32_t taddr = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * BN + c0);
       asm volatile(
@@ -237,7 +237,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc_gemm(const __grid_constant__ 
   // after an abort: wait (bounded) for TMA loads that were issued but never consumed, so no copy is still
   // writing this CTA's shared memory when it exits
   if (threadIdx.x == 0 && *abort_flag) {
-    for (int kb = *n_consumed; kb < *n_loaded; ++kb) mbar_wait(&full[kb % STAGES], (kb / STAGES) & 1);
+    for (int kb = *n_consumed; kb < *n_loaded; ++kb) mbar_wait(&full[kb % stages], (kb / stages) & 1);
   }
   __syncthreads();
   if (warp == 0)
@@ -375,6 +375,27 @@ void tc_init() {
   encode_fn();   // resolve the driver entry point outside any stream capture
 }
 
+// Output tile of a launch.  A K step of a CTA costs about the larger of its six MMAs per 128 rows (N / 2 clocks each, and
+// no less than their operands' 128 bytes a clock from shared memory), the (bm + bn) x 128 bytes it loads at about 40 a
+// clock and SM, and 200 clocks of issue; the launch costs that times its waves of 152.  Measured (us, 256 x 256 -> chosen):
+// tf32x3, n_b 2598 with 2048 right-hand sides (88 tiles of 256 x 256, 143 of 256 x 160) 144 -> 100; three patterns of
+// n_b 1158 with 76 right-hand sides each (15 tiles, mostly padding) 69 -> 25.
+static void tc_tile(const TcProblem& T, const std::vector<int>& busy, int splits, int* bm_out, int* bn_out) {
+  double best = 0.0;
+  for (int bm = BM; bm >= BMH; bm -= BMH)
+    for (int bn = BN; bn >= 32; bn -= 32) {
+      long long ctas = 0;
+      for (int p : busy) ctas += (long long)ceil_div(T.n_b[p], bm) * ceil_div(T.n_rhs[p], bn) * splits;
+      const double mma = 6.0 * (bm / BMH) * std::max(bn / 2.0, 32.0 + bn / 4.0), load = (bm + bn) * 128.0 / 40.0;
+      const double cost = (double)((ctas + 151) / 152) * (200.0 + std::max(mma, load));
+      if (best == 0.0 || cost < best) {
+        best = cost;
+        *bm_out = bm;
+        *bn_out = bn;
+      }
+    }
+}
+
 int tc_ksplits(const TcProblem& T) {
   long long tiles = 0;
   int min_nb = 1 << 30;
@@ -401,6 +422,8 @@ void tc_gemm_split(const TcProblem& T, bool bf16, int* d_error, cudaStream_t s) 
   }
   int splits = tc_ksplits(T);
   if (splits > 1 && (!T.part || T.part_elems < splits * zoff[T.n_pat])) splits = 1;
+  int bm = BM, bn = BN;
+  tc_tile(T, busy, splits, &bm, &bn);
   for (int base = 0; base < (int)busy.size(); base += TC_MAXP) {
     TcParams P;
     std::memset(&P, 0, sizeof(P));
@@ -409,21 +432,23 @@ void tc_gemm_split(const TcProblem& T, bool bf16, int* d_error, cudaStream_t s) 
     int total = 0;
     for (int i = 0; i < P.n_pat; ++i) {
       const int p = busy[base + i];
-      make_map(&P.a_hi[i], T.S_hi[p], T.n_b[p], T.n_b[p], T.lds[p], BM, es);
-      make_map(&P.a_lo[i], T.S_lo[p], T.n_b[p], T.n_b[p], T.lds[p], BM, es);
-      make_map(&P.b_hi[i], T.Y_hi[p], T.n_rhs[p], T.n_b[p], T.ldy[p], BN, es);
-      make_map(&P.b_lo[i], T.Y_lo[p], T.n_rhs[p], T.n_b[p], T.ldy[p], BN, es);
+      make_map(&P.a_hi[i], T.S_hi[p], T.n_b[p], T.n_b[p], T.lds[p], bm, es);
+      make_map(&P.a_lo[i], T.S_lo[p], T.n_b[p], T.n_b[p], T.lds[p], bm, es);
+      make_map(&P.b_hi[i], T.Y_hi[p], T.n_rhs[p], T.n_b[p], T.ldy[p], bn, es);
+      make_map(&P.b_lo[i], T.Y_lo[p], T.n_rhs[p], T.n_b[p], T.ldy[p], bn, es);
       P.Z[i] = T.Z[p];
       P.part[i] = T.part ? T.part + splits * zoff[p] : nullptr;
       P.ldz[i] = T.ldy[p];
       P.n_b[i] = T.n_b[p];
       P.n_rhs[i] = T.n_rhs[p];
-      P.tiles_m[i] = ceil_div(T.n_b[p], BM);
       P.tile_off[i] = total;
-      total += P.tiles_m[i] * ceil_div(T.n_rhs[p], BN);
+      total += ceil_div(T.n_b[p], bm) * ceil_div(T.n_rhs[p], bn);
     }
     P.tile_off[P.n_pat] = total;
     P.splits = splits;
+    P.bm = bm;
+    P.bn = bn;
+    P.stages = std::min(MAX_STAGES, RING_BYTES / (2 * (bm + bn) * ROW_BYTES));
     if (total == 0) continue;
     if (bf16) k_tc_gemm<true><<<total * splits, THREADS, SMEM_BYTES, s>>>(P);
     else k_tc_gemm<false><<<total * splits, THREADS, SMEM_BYTES, s>>>(P);
