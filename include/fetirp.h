@@ -53,8 +53,7 @@ enum {
   FETIRP_PREC_TF32X3 = 2, /* tensor cores (tcgen05 kind::tf32), operands split hi+lo, 3 products, FP32
                              accumulation in TMEM; wrapped in FP64 outer refinement */
   FETIRP_PREC_AUTO = 3,   /* solves only (fetirp_options.precision): per structure, FP32 for latency-bound ones
-                             (every used pattern with n_b <= 512 and n_lambda <= 262144, which then run the
-                             persistent iteration), TF32X3 otherwise; both inside the FP64 refinement */
+                             (every used pattern with n_b <= 512 and n_lambda <= 262144), TF32X3 otherwise; both inside the FP64 refinement */
   FETIRP_PREC_BF16X3 = 4  /* tensor cores (tcgen05 kind::f16 with bf16 operands, twice the tf32 rate), operands
                              split into bf16 pairs (16 significant bits), 3 products, FP32 accumulation in TMEM;
                              operator accurate to ~1e-5 relative; wrapped in FP64 outer refinement.  Rotations of
@@ -88,7 +87,8 @@ typedef struct {
   int64_t history_bytes; /* cap on the two direction-history arrays (a full history restarts the recurrence);
                             0 = half of the free device memory */
   int32_t persistent;  /* 1: structures small enough to be latency-bound (n_lambda <= 262144, k <= 32, FP64 or
-                          FP32 local products) run whole block iterations in one cooperative persistent
+                          FP32 local products with few FMAs, of patterns with n_b < 288 or at most 16 right-hand
+                          sides in all) run whole block iterations in one cooperative persistent
                           launch with bounded grid barriers, stopping on the device at convergence; 0: CUDA
                           graphs of per-phase kernels; default 1 */
   /* Caller-supplied device allocator (for example a framework's caching allocator); both NULL (the default)

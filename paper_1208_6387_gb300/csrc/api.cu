@@ -1993,7 +1993,7 @@ void run_iterations(fetirp_ctx ctx, int prec, int G, bool use_graph, TH* Wh, TH*
 }
 
 // The persistent iteration serves latency-bound structures: FP64 or FP32 local products (SIMT), k <= 32, at
-// most six kernel modes per occurrence, n_lambda up to 262144.
+// most six kernel modes per occurrence, n_lambda up to 262144, small local products.
 bool persist_eligible(fetirp_ctx ctx, int prec) {
   if (!ctx->opt.persistent) return false;
   if (prec != FETIRP_PREC_FP64 && prec != FETIRP_PREC_FP32) return false;
@@ -2003,6 +2003,25 @@ bool persist_eligible(fetirp_ctx ctx, int prec) {
   if (ctx->pc.kind != 0) return false;  // the persistent phases use the unweighted projector
   for (auto& P : ctx->pats)
     if (P->kdim > 6) return false;
+  // Where the local products are more than latency, the per-phase kernels' larger tiles win: the persistent phase
+  // multiplies 16 x 16 tiles and gathers its right-hand sides again for every one of them.  Measured (us per block
+  // iteration, persistent / graphs): FP32 n_b 128, 512 right-hand sides (8.4M FMAs) 125 / 175; 168, 512 193 / 198; 256,
+  // 144 128 / 128; 294, 32 150 / 110; 654, 32 208 / 130; 1158, 243 732 / 315; 256, 1024 (67M) 299 / 265; 168, 2048 (58M)
+  // 539 / 458; 128, 2048 (34M) 346 / 375.  FP64 256, 144 162 / 191; 294, 32 185 / 155; 456, 8 226 / 151; 1158, 243
+  // 1387 / 503; 168, 2048 938 / 1028; 256, 1024 510 / 415.  With at most 16 right-hand sides (one column of those tiles)
+  // the persistent launch stays although the graphs are faster on large patterns (n_b 654, 8: 190 / 123): it is what
+  // options.persistent asks for on the smallest structures.
+  const bool fp64 = prec == FETIRP_PREC_FP64;
+  double fmas = 0.0;
+  int max_nb = 0;
+  const long long n_rhs = (long long)ctx->L.n_occ * ctx->k;
+  for (size_t p = 0; p < ctx->pats.size(); ++p) {
+    if (ctx->use[p].occs.empty()) continue;
+    const double nb = ctx->pats[p]->n_b;
+    fmas += nb * nb * (double)ctx->use[p].occs.size() * ctx->k;
+    max_nb = std::max(max_nb, ctx->pats[p]->n_b);
+  }
+  if ((max_nb >= 288 && n_rhs > 16) || fmas >= (fp64 ? 6.2e7 : 5e7)) return false;
   return persist_ctas(prec == FETIRP_PREC_FP64, ctx->k) > 0;
 }
 

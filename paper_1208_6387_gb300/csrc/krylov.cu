@@ -170,22 +170,41 @@ __global__ void __launch_bounds__(256) k_eta_partial_ds(int n, int k, const doub
             for (int v = 0; v < 4; ++v) ds_madd(ah[u], al[u], bh[v], bl[v], h[u][v], l[u][v]);
         }
     }
-    // add the slices in slice order, 4 outputs of the block at a time
+    // add the slices, 4 outputs of the block at a time, in a fixed order on two levels: a dependent FP64 addition takes
+    // 64 clocks, so an output's slices are shared by as many threads as there are (k = 8: 10 threads of 4 or 5 slices
+    // each instead of one of 42)
+    const int nb4 = nblk * 4, parts = max(1, 256 / nb4);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       __syncthreads();
 #pragma unroll
       for (int v = 0; v < 4; ++v) red[tid][v] = act ? ds2d(h[u][v], l[u][v]) : 0.0;
       __syncthreads();
-      if (act && sl == 0) {
-        const int i = i0 + u;
+      if (nb4 > 256) {   // more outputs than threads: at most three slices, added by the first's thread
+        if (act && sl == 0) {
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          double acc = red[tid][v];
-          for (int q = 1; q < slices; ++q) acc += red[tid + q * nblk][v];
-          const int j = j0 + v;
-          if (i < k && j <= k) partial[(size_t)blockIdx.x * nout + (size_t)i * (k + 1) + j] = acc;
+          for (int v = 0; v < 4; ++v) {
+            double acc = red[tid][v];
+            for (int q = 1; q < slices; ++q) acc += red[tid + q * nblk][v];
+            const int i = i0 + u, j = j0 + v;
+            if (i < k && j <= k) partial[(size_t)blockIdx.x * nout + (size_t)i * (k + 1) + j] = acc;
+          }
         }
+        continue;
+      }
+      double acc = 0.0;
+      const int o = tid % nb4, pt = tid / nb4;   // output (block, column) of this thread, its share of the slices
+      if (pt < parts) {
+        const int q0 = pt * slices / parts, q1 = (pt + 1) * slices / parts;
+        for (int q = q0; q < q1; ++q) acc += red[(o >> 2) + q * nblk][o & 3];
+      }
+      __syncthreads();
+      if (pt < parts) (&red[0][0])[tid] = acc;
+      __syncthreads();
+      if (tid < nb4) {
+        for (int q = 1; q < parts; ++q) acc += (&red[0][0])[tid + q * nb4];
+        const int i = (o >> 2) / bj * 4 + u, j = (o >> 2) % bj * 4 + (o & 3);
+        if (i < k && j <= k) partial[(size_t)blockIdx.x * nout + (size_t)i * (k + 1) + j] = acc;
       }
     }
   }
@@ -588,14 +607,17 @@ __global__ void k_eta_group_sums(int nout, int chunks, const double* __restrict_
 
 int eta_partials(int n, int k, const double* W, const double* Q, const double* r, DBuf<double>& partial,
                  cudaStream_t s, bool ds, int* n_read) {
-  const bool small = ds && k == 4;
+  const bool small = ds && k <= 4;
   // narrow blocks: one CTA per SM, a few thousand rows each (every thread sums several rows before the
   // per-CTA reduction); otherwise up to 608 chunks of >= 256 rows
   const int chunks = small ? std::max(1, std::min(152, ceil_div(n, 1024))) : eta_chunks(n);
   const int rows = ceil_div(n, chunks);
   const int nout = k * (k + 1);
   partial.ensure((size_t)(chunks + ETA_GROUPS) * nout);
-  if (small) k_eta_small_ds<4><<<chunks, 256, 0, s>>>(n, W, Q, r, rows, partial.p);
+  if (small && k == 4) k_eta_small_ds<4><<<chunks, 256, 0, s>>>(n, W, Q, r, rows, partial.p);
+  else if (small && k == 3) k_eta_small_ds<3><<<chunks, 256, 0, s>>>(n, W, Q, r, rows, partial.p);
+  else if (small && k == 2) k_eta_small_ds<2><<<chunks, 256, 0, s>>>(n, W, Q, r, rows, partial.p);
+  else if (small) k_eta_small_ds<1><<<chunks, 256, 0, s>>>(n, W, Q, r, rows, partial.p);
   else if (ds) k_eta_partial_ds<<<chunks, 256, 0, s>>>(n, k, W, Q, r, rows, partial.p);
   else k_eta_partial<<<chunks, 256, 0, s>>>(n, k, W, Q, r, rows, partial.p);
   FETIRP_LAUNCH_CHECK();
