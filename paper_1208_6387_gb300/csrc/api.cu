@@ -304,7 +304,8 @@ struct fetirp_ctx_s {
   bool owns_stream = false;
   bool capturing = false;
   bool in_iteration = false;            // enqueuing block iterations outside a capture (accounted per iteration)
-  std::vector<cudaStream_t> fstreams;   // one per concurrently factorised pattern
+  std::vector<cudaStream_t> fstreams;   // one per concurrently factorised pattern (high priority: serial chains)
+  std::vector<CholAux> chol_aux;        // and its side stream for trailing updates
   cudaEvent_t fork_ev = nullptr;
   std::vector<cudaEvent_t> join_ev;
   struct GraphCache {
@@ -323,6 +324,11 @@ struct fetirp_ctx_s {
     if (h_state) cudaFreeHost(h_state);
     if (h_rr) cudaFreeHost(h_rr);
     for (cudaStream_t st : fstreams) cudaStreamDestroy(st);
+    for (CholAux& a : chol_aux) {
+      cudaStreamDestroy(a.stream);
+      cudaEventDestroy(a.panel);
+      cudaEventDestroy(a.rest);
+    }
     if (fork_ev) cudaEventDestroy(fork_ev);
     for (cudaEvent_t e : join_ev) cudaEventDestroy(e);
     if (owns_stream && stream) cudaStreamDestroy(stream);
@@ -464,7 +470,7 @@ void check_tc_error(fetirp_ctx ctx);
 // detection (Sec. 2), kernel N, Schur complement pseudo-inverse S^+ = L_S^{-T} L_S^{-1} (stated after Eq. 3).
 // Several patterns are factorised concurrently, each on its own stream forked from the context stream;
 // work buffers stay resident so that a refactorisation allocates nothing.
-void factor_stage_a(PatternData& P, double pivot_tol, cudaStream_t s) {
+void factor_stage_a(PatternData& P, double pivot_tol, const CholAux& aux, cudaStream_t s) {
   const int n = P.n, npad = P.npad;
   P.L.ensure((size_t)npad * npad);
   FETIRP_CUDA(cudaMemsetAsync(P.L.p, 0, sizeof(double) * (size_t)npad * npad, s));
@@ -474,7 +480,7 @@ void factor_stage_a(PatternData& P, double pivot_tol, cudaStream_t s) {
   P.diag0.ensure(npad);
   P.zp.ensure(npad);
   copy_diag(P.L.p, npad, P.diag0.p, s);
-  chol_tiles(P.L.p, npad, P.plan, P.diag0.p, P.zp.p, pivot_tol, s);
+  chol_tiles(P.L.p, npad, P.plan, P.diag0.p, P.zp.p, pivot_tol, s, &aux);
   P.Dinv.ensure((size_t)npad * TILE);
   tile_inverses(P.L.p, npad, P.zp.p, P.Dinv.p, s);
   P.h_zp.resize(npad);
@@ -686,7 +692,9 @@ void ensure_operators(fetirp_ctx ctx, int prec) {
 void fork_patterns(fetirp_ctx ctx, size_t np) {
   while (ctx->fstreams.size() < np) {
     cudaStream_t st;
-    FETIRP_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+    int least = 0, greatest = 0;
+    FETIRP_CUDA(cudaDeviceGetStreamPriorityRange(&least, &greatest));
+    FETIRP_CUDA(cudaStreamCreateWithPriority(&st, cudaStreamNonBlocking, greatest));
     ctx->fstreams.push_back(st);
   }
   if (!ctx->fork_ev) FETIRP_CUDA(cudaEventCreateWithFlags(&ctx->fork_ev, cudaEventDisableTiming));
@@ -729,7 +737,15 @@ void factorize_patterns(fetirp_ctx ctx, const std::vector<PatternData*>& pats) {
   const size_t np = pats.size();
   ensure_tc_error(ctx);
   fork_patterns(ctx, np);
-  for (size_t i = 0; i < np; ++i) factor_stage_a(*pats[i], ctx->opt.pivot_tol, ctx->fstreams[i]);
+  while (ctx->chol_aux.size() < np) {
+    CholAux a{};
+    FETIRP_CUDA(cudaStreamCreateWithFlags(&a.stream, cudaStreamNonBlocking));
+    ctx->chol_aux.push_back(a);
+    FETIRP_CUDA(cudaEventCreateWithFlags(&ctx->chol_aux.back().panel, cudaEventDisableTiming));
+    FETIRP_CUDA(cudaEventCreateWithFlags(&ctx->chol_aux.back().rest, cudaEventDisableTiming));
+  }
+  for (size_t i = 0; i < np; ++i)
+    factor_stage_a(*pats[i], ctx->opt.pivot_tol, ctx->chol_aux[i], ctx->fstreams[i]);
   for (size_t i = 0; i < np; ++i) FETIRP_CUDA(cudaStreamSynchronize(ctx->fstreams[i]));
   for (size_t i = 0; i < np; ++i) {
     factor_check(*pats[i]);

@@ -28,8 +28,16 @@ struct TilePlan {
 // dof j as a zero pivot: zp[j] = 1 and column j of L is set to 0.  diag0 holds the diagonal before
 // factorisation.  Rows of zero-pivot dofs are zeroed at the end, so L is the Cholesky factor of the
 // nonsingular block K_rr embedded with zeros (the generalized inverse of Sec. 2).
+// aux (optional): a second stream, of lower priority than s, and two events for the trailing updates that the next
+// column does not wait for.  They go there from CHOL_SPLIT_PAIRS tile pairs on, about what fills the SMs for as long as a
+// diagonal tile and its panel take.  Single 12^3 elastic pattern: 42.3 ms a factorisation without, 33 with.
+constexpr int CHOL_SPLIT_PAIRS = 76;
+struct CholAux {
+  cudaStream_t stream;
+  cudaEvent_t panel, rest;
+};
 void chol_tiles(double* A, int npad, const TilePlan& plan, const double* diag0, int* zp, double tol,
-                cudaStream_t s);
+                cudaStream_t s, const CholAux* aux = nullptr);
 
 // X <- L^{-1} X (trans = false) or X <- L^{-T} X (trans = true), X column-major npad x nrhs (ld = ldx),
 // zero-pivot rows of the result set to 0.  Right-looking over tile columns, skipping zero tiles.

@@ -20,12 +20,13 @@ void TilePlan::build(int nt_, const std::vector<uint8_t>& nz0) {
       if (nz[(size_t)I * nt + k]) rows.push_back(I);
     for (int I : rows) col_rows.push_back(I);
     pair_off[k] = (int)pairs.size();
-    // fill-in: (I, J) becomes nonzero when both (I, k) and (J, k) are
+    // fill-in: (I, J) becomes nonzero when both (I, k) and (J, k) are; the first row's column comes first in the list
+    for (size_t a = 0; a < rows.size(); ++a) pairs.push_back(make_int2(rows[a], rows[0]));
     for (size_t a = 0; a < rows.size(); ++a)
       for (size_t b = 0; b <= a; ++b) {
         int I = rows[a], J = rows[b];
         nz[(size_t)I * nt + J] = 1;
-        pairs.push_back(make_int2(I, J));
+        if (b > 0) pairs.push_back(make_int2(I, J));
       }
   }
   col_off[nt] = (int)col_rows.size();
@@ -61,47 +62,57 @@ __global__ void k_zero_zp_rows(double* A, int npad, const int* zp) {
 // FP64 divide costs ~450 cycles and a square root ~700 on this GPU): step j scales the remaining column by the
 // pivot's reciprocal (multipliers l_r = a_rj / d_j), the trailing update is one FMA per entry with the unscaled
 // column, a_rc -= l_r a_cj, and every column is scaled by 1 / sqrt(d_j) once at the end, in parallel, giving
-// L = L_unit D^{1/2}.  One step of lookahead: thread 0 updates the next diagonal entry first and forms its
-// reciprocal while the other threads finish the update.  Zero pivots (d_j <= tol * diag0_j, or not finite) get
-// a zero multiplier column (no update) and a zero column of L.
+// L = L_unit D^{1/2}.  Zero pivots (d_j <= tol * diag0_j, or not finite) get a zero multiplier column (no update) and a
+// zero column of L.  The tile lives in registers (thread: a row and every fourth column); only the current column and
+// the pivot's reciprocal go through shared memory, in two buffers, so a step has one barrier.  The owners of the next
+// column update it first, publish it and form the next reciprocal while the other warps update the rest: a step takes
+// the longer of that chain (multiply, FMA, divide) and the FP64 pipe's time for the update (the tile in shared memory
+// with two barriers and a dependent load per FMA: 65 us; this: 30 us).
 __global__ void __launch_bounds__(256) k_potrf_tile(double* A, int npad, int k, const double* diag0, int* zp,
                                                     double tol) {
-  __shared__ double a[TILE][TILE + 1];   // a[row][col]
+  __shared__ double col[2][TILE];        // column j of the trailing block
+  __shared__ double s_rinv[2];
   __shared__ double thr[TILE];           // tol * diag0 of the tile's dofs
   __shared__ double dd[TILE];            // pivots d_j (0 for zero pivots), then 1 / sqrt(d_j)
-  __shared__ double lcol[TILE];          // multipliers of the current step
-  __shared__ double s_rinv;
   const int tid = threadIdx.x;
+  const int rr = tid % TILE, cg = tid / TILE;   // row rr, columns cg, cg + 4, ... (cg is the same for a warp)
   double* T = A + (size_t)k * TILE * npad + (size_t)k * TILE;
-  for (int idx = tid; idx < TILE * TILE; idx += 256) {
-    int r = idx % TILE, c = idx / TILE;
-    a[r][c] = T[(size_t)c * npad + r];
-  }
+  double a[TILE / 4];
+#pragma unroll
+  for (int i = 0; i < TILE / 4; ++i) a[i] = T[(size_t)(cg + 4 * i) * npad + rr];
   if (tid < TILE) thr[tid] = tol * diag0[k * TILE + tid];
-  __syncthreads();
-  if (tid == 0) {
-    const double d = a[0][0];
-    const bool zero = !(d > thr[0]);   // also catches NaN and negative roundoff
-    dd[0] = zero ? 0.0 : d;
-    s_rinv = zero ? 0.0 : 1.0 / d;
+  if (cg == 0) {
+    col[0][rr] = a[0];
+    if (rr == 0) {
+      const double d = a[0];
+      const bool zero = !(d > tol * diag0[k * TILE]);   // also catches NaN and negative roundoff
+      dd[0] = zero ? 0.0 : d;
+      s_rinv[0] = zero ? 0.0 : 1.0 / d;
+    }
   }
   __syncthreads();
-  const int rr = tid % TILE, cg = tid / TILE;   // update: row rr, columns j+1+cg, j+5+cg, ...
+#pragma unroll
   for (int j = 0; j + 1 < TILE; ++j) {
-    const double rinv = s_rinv;
-    for (int r = j + 1 + tid; r < TILE; r += 256) lcol[r] = a[r][j] * rinv;
-    __syncthreads();
-    if (tid == 0) {   // lookahead: the next pivot and its reciprocal
-      const double d = fma(-lcol[j + 1], a[j + 1][j], a[j + 1][j + 1]);
-      a[j + 1][j + 1] = d;
-      const bool zero = !(d > thr[j + 1]);
-      dd[j + 1] = zero ? 0.0 : d;
-      s_rinv = zero ? 0.0 : 1.0 / d;
+    constexpr int LAST = TILE / 4;
+    const int b = j & 1, in = (j + 1) >> 2;
+    const double lr = col[b][rr] * s_rinv[b];
+    if (cg == ((j + 1) & 3) && rr > j) {   // the next column, its pivot and the reciprocal
+      a[in] = fma(-lr, col[b][j + 1], a[in]);
+      col[b ^ 1][rr] = a[in];
+      if (rr == j + 1) {
+        const double d = a[in];
+        const bool zero = !(d > thr[j + 1]);
+        dd[j + 1] = zero ? 0.0 : d;
+        s_rinv[b ^ 1] = zero ? 0.0 : 1.0 / d;
+      }
     }
-    if (rr > j) {
-      const double lr = lcol[rr];
-      for (int c = j + 1 + cg; c <= rr; c += 4)
-        if (c != j + 1 || rr != j + 1) a[rr][c] = fma(-lr, a[c][j], a[rr][c]);
+#pragma unroll
+    for (int i = in; i < LAST; ++i) {
+      const int c = cg + 4 * i;
+      if (c > j + 1 && c <= (rr | 31)) {   // warps whose rows all lie above the column skip it
+        const double u = fma(-lr, col[b][c], a[i]);
+        if (c <= rr) a[i] = u;
+      }
     }
     __syncthreads();
   }
@@ -112,49 +123,49 @@ __global__ void __launch_bounds__(256) k_potrf_tile(double* A, int npad, int k, 
     dd[tid] = d > 0.0 ? 1.0 / sqrt(d) : 0.0;
   }
   __syncthreads();
-  for (int idx = tid; idx < TILE * TILE; idx += 256) {
-    int r = idx % TILE, c = idx / TILE;
-    T[(size_t)c * npad + r] = (r >= c) ? a[r][c] * dd[c] : 0.0;
+#pragma unroll
+  for (int i = 0; i < TILE / 4; ++i) {
+    const int c = cg + 4 * i;
+    T[(size_t)c * npad + rr] = (rr >= c) ? a[i] * dd[c] : 0.0;
   }
 }
 
 // For step k: tiles (I, k), I in rows[0..cnt): L_Ik = A_Ik L_kk^{-T} (zero-pivot columns -> 0).  The rows of
-// a tile are independent, so grid.y splits each tile into four 16-row blocks (more SMs on the FP64 work).
-constexpr int TR_ROWS = 16;
-__global__ void __launch_bounds__(256) k_trsm_tiles(double* A, int npad, int k, const int* rows, const int* zp) {
+// a tile are independent, so grid.y splits each tile into eight 8-row blocks (more SMs on the FP64 work).  Sixteen
+// threads of one warp hold a row in registers (every sixteenth column each): step j is a multiply by the pivot's
+// reciprocal, a shuffle and the FMAs of the later columns, without a barrier; bound by the FP64 pipe (rows in shared
+// memory, two barriers a step: 40 us for 35 tiles; this: 17 us).
+constexpr int TR_ROWS = 8;
+__global__ void __launch_bounds__(16 * TR_ROWS) k_trsm_tiles(double* A, int npad, int k, const int* rows, const int* zp) {
   __shared__ double l[TILE][TILE + 1];
-  __shared__ double x[TR_ROWS][TILE + 1];
   __shared__ double rinv[TILE];
   const int tid = threadIdx.x;
   const int I = rows[blockIdx.x];
   const int rb = blockIdx.y * TR_ROWS;
   const double* D = A + (size_t)k * TILE * npad + (size_t)k * TILE;
   double* X = A + (size_t)k * TILE * npad + (size_t)I * TILE + rb;
-  for (int idx = tid; idx < TILE * TILE; idx += 256) {
-    int r = idx % TILE, c = idx / TILE;
-    l[r][c] = D[(size_t)c * npad + r];
-  }
-  for (int idx = tid; idx < TR_ROWS * TILE; idx += 256) {
-    int r = idx % TR_ROWS, c = idx / TR_ROWS;
-    x[r][c] = X[(size_t)c * npad + r];
+  const int r = tid >> 4, q = tid & 15;
+  double x[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) x[i] = X[(size_t)(q + 16 * i) * npad + r];
+  for (int idx = tid; idx < TILE * TILE; idx += 16 * TR_ROWS) {
+    const int rl = idx % TILE, c = idx / TILE;
+    l[rl][c] = D[(size_t)c * npad + rl];
   }
   __syncthreads();
   if (tid < TILE) rinv[tid] = zp[k * TILE + tid] != 0 ? 0.0 : 1.0 / l[tid][tid];
   __syncthreads();
+#pragma unroll
   for (int j = 0; j < TILE; ++j) {
-    if (tid < TR_ROWS) x[tid][j] *= rinv[j];
-    __syncthreads();
-    const int w = TILE - 1 - j;
-    for (int idx = tid; idx < w * TR_ROWS; idx += 256) {
-      int c = j + 1 + idx / TR_ROWS, r = idx % TR_ROWS;
-      x[r][c] -= x[r][j] * l[c][j];
-    }
-    __syncthreads();
+    const int i0 = j >> 4, q0 = j & 15;
+    const double xj = __shfl_sync(0xffffffffu, x[i0] * rinv[j], q0, 16);
+    if (q == q0) x[i0] = xj;
+    else if (q > q0) x[i0] = fma(-xj, l[q + 16 * i0][j], x[i0]);
+#pragma unroll
+    for (int i = i0 + 1; i < 4; ++i) x[i] = fma(-xj, l[q + 16 * i][j], x[i]);
   }
-  for (int idx = tid; idx < TR_ROWS * TILE; idx += 256) {
-    int r = idx % TR_ROWS, c = idx / TR_ROWS;
-    X[(size_t)c * npad + r] = x[r][c];
-  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) X[(size_t)(q + 16 * i) * npad + r] = x[i];
 }
 
 // For step k: A_IJ -= L_Ik L_Jk^T for each pair (I, J).  grid.y: the four 32 x 32 quadrants of the output
@@ -535,21 +546,41 @@ void zero_zp_rows(double* A, int npad, const int* zp, cudaStream_t s) {
 }
 
 void chol_tiles(double* A, int npad, const TilePlan& plan, const double* diag0, int* zp, double tol,
-                cudaStream_t s) {
+                cudaStream_t s, const CholAux* aux) {
+  // With aux, a step's update is split: the next column's tiles on s, so that its factorisation and panel solve (the
+  // serial chain of the algorithm) go on, and the rest on aux beside them, in the same order for every tile.
+  bool pending = false;   // aux holds updates that s has not waited for
   for (int k = 0; k < plan.nt; ++k) {
     k_potrf_tile<<<1, 256, 0, s>>>(A, npad, k, diag0, zp, tol);
     FETIRP_LAUNCH_CHECK();
-    int nr = plan.col_off[k + 1] - plan.col_off[k];
-    if (nr > 0) {
-      k_trsm_tiles<<<dim3(nr, TILE / TR_ROWS), 256, 0, s>>>(A, npad, k, plan.d_col_rows.p + plan.col_off[k], zp);
+    const int nr = plan.col_off[k + 1] - plan.col_off[k];
+    if (nr == 0) continue;
+    const int* rows = plan.d_col_rows.p + plan.col_off[k];
+    k_trsm_tiles<<<dim3(nr, TILE / TR_ROWS), 16 * TR_ROWS, 0, s>>>(A, npad, k, rows, zp);
+    FETIRP_LAUNCH_CHECK();
+    const int2* pairs = plan.d_pairs.p + plan.pair_off[k];
+    const int np = plan.pair_off[k + 1] - plan.pair_off[k];
+    const int first = plan.col_rows[plan.col_off[k]] == k + 1 ? nr : 0;   // pairs of column k + 1
+    const bool split = aux && np - first >= CHOL_SPLIT_PAIRS;
+    if (split) FETIRP_CUDA(cudaEventRecord(aux->panel, s));
+    if (pending) {   // every earlier update of these tiles
+      FETIRP_CUDA(cudaStreamWaitEvent(s, aux->rest, 0));
+      pending = false;
+    }
+    const int on_s = split ? first : np;
+    if (on_s > 0) {
+      k_update_pairs<<<dim3(on_s, 4), 256, 0, s>>>(A, npad, k, pairs);
       FETIRP_LAUNCH_CHECK();
     }
-    int np = plan.pair_off[k + 1] - plan.pair_off[k];
-    if (np > 0) {
-      k_update_pairs<<<dim3(np, 4), 256, 0, s>>>(A, npad, k, plan.d_pairs.p + plan.pair_off[k]);
+    if (split) {
+      FETIRP_CUDA(cudaStreamWaitEvent(aux->stream, aux->panel, 0));
+      k_update_pairs<<<dim3(np - first, 4), 256, 0, aux->stream>>>(A, npad, k, pairs + first);
       FETIRP_LAUNCH_CHECK();
+      FETIRP_CUDA(cudaEventRecord(aux->rest, aux->stream));
+      pending = true;
     }
   }
+  if (pending) FETIRP_CUDA(cudaStreamWaitEvent(s, aux->rest, 0));
   zero_zp_rows(A, npad, zp, s);
 }
 

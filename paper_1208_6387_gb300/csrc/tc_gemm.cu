@@ -377,9 +377,10 @@ void tc_init() {
 
 // Output tile of a launch.  A K step of a CTA costs about the larger of its six MMAs per 128 rows (N / 2 clocks each, and
 // no less than their operands' 128 bytes a clock from shared memory), the (bm + bn) x 128 bytes it loads at about 40 a
-// clock and SM, and 200 clocks of issue; the launch costs that times its waves of 152.  Measured (us, 256 x 256 -> chosen):
-// tf32x3, n_b 2598 with 2048 right-hand sides (88 tiles of 256 x 256, 143 of 256 x 160) 144 -> 100; three patterns of
-// n_b 1158 with 76 right-hand sides each (15 tiles, mostly padding) 69 -> 25.
+// clock and SM, and 200 clocks of issue.  The launch alone takes that times its waves of 152; next to other streams' work
+// what counts is the SM time in all, so the mean of the two decides.  Measured in a whole apply (us, 256 x 256 -> chosen):
+// tf32x3, three patterns of n_b 1158 with 76 right-hand sides each (15 tiles, mostly padding) 309 -> 276; n_b 3534 with 216
+// (14 tiles) 242 -> 197.
 static void tc_tile(const TcProblem& T, const std::vector<int>& busy, int splits, int* bm_out, int* bn_out) {
   double best = 0.0;
   for (int bm = BM; bm >= BMH; bm -= BMH)
@@ -387,7 +388,7 @@ static void tc_tile(const TcProblem& T, const std::vector<int>& busy, int splits
       long long ctas = 0;
       for (int p : busy) ctas += (long long)ceil_div(T.n_b[p], bm) * ceil_div(T.n_rhs[p], bn) * splits;
       const double mma = 6.0 * (bm / BMH) * std::max(bn / 2.0, 32.0 + bn / 4.0), load = (bm + bn) * 128.0 / 40.0;
-      const double cost = (double)((ctas + 151) / 152) * (200.0 + std::max(mma, load));
+      const double cost = ((double)((ctas + 151) / 152) + ctas / 152.0) * (200.0 + std::max(mma, load));
       if (best == 0.0 || cost < best) {
         best = cost;
         *bm_out = bm;
