@@ -62,56 +62,64 @@ __global__ void k_zero_zp_rows(double* A, int npad, const int* zp) {
 // FP64 divide costs ~450 cycles and a square root ~700 on this GPU): step j scales the remaining column by the
 // pivot's reciprocal (multipliers l_r = a_rj / d_j), the trailing update is one FMA per entry with the unscaled
 // column, a_rc -= l_r a_cj, and every column is scaled by 1 / sqrt(d_j) once at the end, in parallel, giving
-// L = L_unit D^{1/2}.  Zero pivots (d_j <= tol * diag0_j, or not finite) get a zero multiplier column (no update) and a
-// zero column of L.  The tile lives in registers (thread: a row and every fourth column); only the current column and
-// the pivot's reciprocal go through shared memory, in two buffers, so a step has one barrier.  The owners of the next
-// column update it first, publish it and form the next reciprocal while the other warps update the rest: a step takes
-// the longer of that chain (multiply, FMA, divide) and the FP64 pipe's time for the update (the tile in shared memory
-// with two barriers and a dependent load per FMA: 65 us; this: 30 us).
+// L = L_unit D^{1/2}.  One step of lookahead: thread 0 updates the next diagonal entry first and forms its
+// reciprocal while the other threads finish the update.  Zero pivots (d_j <= tol * diag0_j, or not finite) get
+// a zero multiplier column (no update) and a zero column of L.  The step's column is copied beside the tile, so that a
+// thread's loads of four entries do not wait for its stores, and a thread takes four entries at a time.
 __global__ void __launch_bounds__(256) k_potrf_tile(double* A, int npad, int k, const double* diag0, int* zp,
                                                     double tol) {
-  __shared__ double col[2][TILE];        // column j of the trailing block
-  __shared__ double s_rinv[2];
+  __shared__ double a[TILE][TILE + 1];   // a[row][col]
   __shared__ double thr[TILE];           // tol * diag0 of the tile's dofs
   __shared__ double dd[TILE];            // pivots d_j (0 for zero pivots), then 1 / sqrt(d_j)
+  __shared__ double lcol[TILE];          // multipliers of the current step
+  __shared__ double ccol[TILE];          // its unscaled column
+  __shared__ double s_rinv;
   const int tid = threadIdx.x;
-  const int rr = tid % TILE, cg = tid / TILE;   // row rr, columns cg, cg + 4, ... (cg is the same for a warp)
   double* T = A + (size_t)k * TILE * npad + (size_t)k * TILE;
-  double a[TILE / 4];
-#pragma unroll
-  for (int i = 0; i < TILE / 4; ++i) a[i] = T[(size_t)(cg + 4 * i) * npad + rr];
+  for (int idx = tid; idx < TILE * TILE; idx += 256) {
+    int r = idx % TILE, c = idx / TILE;
+    a[r][c] = T[(size_t)c * npad + r];
+  }
   if (tid < TILE) thr[tid] = tol * diag0[k * TILE + tid];
-  if (cg == 0) {
-    col[0][rr] = a[0];
-    if (rr == 0) {
-      const double d = a[0];
-      const bool zero = !(d > tol * diag0[k * TILE]);   // also catches NaN and negative roundoff
-      dd[0] = zero ? 0.0 : d;
-      s_rinv[0] = zero ? 0.0 : 1.0 / d;
-    }
+  __syncthreads();
+  if (tid == 0) {
+    const double d = a[0][0];
+    const bool zero = !(d > thr[0]);   // also catches NaN and negative roundoff
+    dd[0] = zero ? 0.0 : d;
+    s_rinv = zero ? 0.0 : 1.0 / d;
   }
   __syncthreads();
-#pragma unroll
+  const int rr = tid % TILE, cg = tid / TILE;   // update: row rr, columns j+1+cg, j+5+cg, ...
   for (int j = 0; j + 1 < TILE; ++j) {
-    constexpr int LAST = TILE / 4;
-    const int b = j & 1, in = (j + 1) >> 2;
-    const double lr = col[b][rr] * s_rinv[b];
-    if (cg == ((j + 1) & 3) && rr > j) {   // the next column, its pivot and the reciprocal
-      a[in] = fma(-lr, col[b][j + 1], a[in]);
-      col[b ^ 1][rr] = a[in];
-      if (rr == j + 1) {
-        const double d = a[in];
-        const bool zero = !(d > thr[j + 1]);
-        dd[j + 1] = zero ? 0.0 : d;
-        s_rinv[b ^ 1] = zero ? 0.0 : 1.0 / d;
-      }
+    const double rinv = s_rinv;
+    if (tid > j && tid < TILE) {
+      const double v = a[tid][j];
+      ccol[tid] = v;
+      lcol[tid] = v * rinv;
     }
+    __syncthreads();
+    if (tid == 0) {   // lookahead: the next pivot and its reciprocal
+      const double d = fma(-lcol[j + 1], ccol[j + 1], a[j + 1][j + 1]);
+      a[j + 1][j + 1] = d;
+      const bool zero = !(d > thr[j + 1]);
+      dd[j + 1] = zero ? 0.0 : d;
+      s_rinv = zero ? 0.0 : 1.0 / d;
+    }
+    if (rr > j) {
+      const double lr = lcol[rr];
+      const bool skip = rr == j + 1;      // its only entry is the next diagonal one
+      double* ar = a[rr];
+      for (int c = j + 1 + cg; c <= rr && !skip; c += 16) {
+        double v[4], w[4];
 #pragma unroll
-    for (int i = in; i < LAST; ++i) {
-      const int c = cg + 4 * i;
-      if (c > j + 1 && c <= (rr | 31)) {   // warps whose rows all lie above the column skip it
-        const double u = fma(-lr, col[b][c], a[i]);
-        if (c <= rr) a[i] = u;
+        for (int u = 0; u < 4; ++u) {
+          const int cu = min(c + 4 * u, TILE - 1);
+          v[u] = ar[cu];
+          w[u] = ccol[cu];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (c + 4 * u <= rr) ar[c + 4 * u] = fma(-lr, w[u], v[u]);
       }
     }
     __syncthreads();
@@ -123,10 +131,9 @@ __global__ void __launch_bounds__(256) k_potrf_tile(double* A, int npad, int k, 
     dd[tid] = d > 0.0 ? 1.0 / sqrt(d) : 0.0;
   }
   __syncthreads();
-#pragma unroll
-  for (int i = 0; i < TILE / 4; ++i) {
-    const int c = cg + 4 * i;
-    T[(size_t)c * npad + rr] = (rr >= c) ? a[i] * dd[c] : 0.0;
+  for (int idx = tid; idx < TILE * TILE; idx += 256) {
+    int r = idx % TILE, c = idx / TILE;
+    T[(size_t)c * npad + r] = (r >= c) ? a[r][c] * dd[c] : 0.0;
   }
 }
 
