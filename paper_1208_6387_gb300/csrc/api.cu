@@ -2088,6 +2088,12 @@ PersistArgs persist_args(fetirp_ctx ctx, bool fp64, TH* Wh, TH* Qh) {
   A.Ginv = ctx->Ginv.p; A.Xc = ctx->Xc.p; A.Ac = ctx->Ac.p;
   // history splits sized for the persistent grid (about one item per CTA; never more than tu_part holds)
   A.tu_splits = std::max(1, std::min(tall_update_splits(nl, (int)ctx->hist_cap), A.ncta / ceil_div(nl, 64)));
+  // one row per thread: the longest histories leave every split at least 64 directions
+  A.tu_vsplits = 0;
+  if (!fp64 && (k == 4 || k == 8 || k == 16 || k == 32)) {
+    A.tu_vsplits = (int)std::max<long long>(1, std::min<long long>(A.ncta / ceil_div(nl, 1024 / k), ctx->hist_cap / 64));
+    ctx->tu_part.ensure((size_t)A.tu_vsplits * nl * k);
+  }
   A.tu_part = ctx->tu_part.p; A.tu_tickets = ctx->tu_tickets.p;
   const int nout = k * (k + 1);
   ctx->pers_eta.ensure((size_t)(A.ncta + 64) * nout);

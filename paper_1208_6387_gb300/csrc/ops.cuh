@@ -238,8 +238,9 @@ struct PersistArgs {
   const double* Ginv;
   double* Xc;
   double* Ac;
-  // history update
+  // history update; tu_vsplits > 0: the one-row-per-thread form with that many history splits (FP32, k = 4, 8, 16, 32)
   int tu_splits;
+  int tu_vsplits;
   void* tu_part;
   unsigned* tu_tickets;
   // eta and the normalisation

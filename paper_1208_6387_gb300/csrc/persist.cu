@@ -184,10 +184,16 @@ __device__ void phase_gtv(const PersistArgs& A, unsigned char* smem) {
   for (int it = blockIdx.x; it < items; it += A.ncta) gtv_item<TL, from_split>(A, it, smem);
 }
 
-// C partials of Q_h^T S(r).  Item: (128 history columns, group, 128-row chunk); the chunk's (row, w r[row]) pairs
+// C partials of Q_h^T S(r).  Item: (some tiles of 128 history columns, group, 128-row chunk); the chunk's (row, w r[row]) pairs
 // are staged in shared memory, the 8 warps take every 8th row, each lane four columns, the warp sums are added
 // in warp order (deterministic); FP32 history: double-single sums on the FP32 pipe (see the split Gram kernel).
 constexpr int P_GC = 128;
+// Parts that the history columns of a (group, row chunk) are cut into: about an item per CTA, so that a chunk's rows,
+// two dependent loads away, are staged once for several column tiles
+__device__ __forceinline__ int gram_parts(const PersistArgs& A, int a) {
+  const int ctiles = (a + P_GC - 1) / P_GC;
+  return min(ctiles, max(1, A.ncta / max(1, A.k * A.gs_chunks)));
+}
 template <typename TH>
 __device__ void gram_item(const PersistArgs& A, int a, int it, unsigned char* smem) {
   int* srow = reinterpret_cast<int*>(smem);
@@ -197,9 +203,9 @@ __device__ void gram_item(const PersistArgs& A, int a, int it, unsigned char* sm
   double (*red)[P_GC] = reinterpret_cast<double (*)[P_GC]>(smem + 512 + 1024 + 1024);
   const TH* Qh = (const TH*)A.Qh;
   const int k = A.k;   // also the history block width
-  const int ctiles = (a + P_GC - 1) / P_GC;
+  const int ctiles = (a + P_GC - 1) / P_GC, cparts = gram_parts(A, a);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int ct = it % ctiles, rest = it / ctiles, g = rest % k, ch = rest / k;
+  const int cp = it % cparts, rest = it / cparts, g = rest % k, ch = rest / k;
   const int e0 = A.grp_ptr[g] + ch * P_GS_ROWS, e1 = min(A.grp_ptr[g + 1], e0 + P_GS_ROWS);
   const int cnt = max(0, e1 - e0);
   __syncthreads();
@@ -211,6 +217,7 @@ __device__ void gram_item(const PersistArgs& A, int a, int it, unsigned char* sm
     d2ds(v, swh[tid], swl[tid]);
   }
   __syncthreads();
+  for (int ct = cp * ctiles / cparts; ct < (cp + 1) * ctiles / cparts; ++ct) {
   bool ok[4];
   const TH* qp[4];
 #pragma unroll
@@ -220,7 +227,39 @@ __device__ void gram_item(const PersistArgs& A, int a, int it, unsigned char* sm
     qp[u] = Qh + hist_col(ok[u] ? c : 0, A.n, k);
   }
   double res[4];
-  if (sizeof(TH) == 4) {
+  // history widths in fours: a lane takes four consecutive columns, one 16-byte load per row, eight rows in flight
+  const bool vec = sizeof(TH) == 4 && k % 4 == 0;
+  if (vec) {
+    float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
+    const int c = ct * P_GC + 4 * lane;   // a is a multiple of k: the four columns are stored together or not at all
+    const float* q4 = (const float*)Qh + hist_col(c < a ? c : 0, A.n, k);
+    if (c < a) {
+#pragma unroll 1
+      for (int i0 = warp; i0 < cnt; i0 += 64) {
+        float4 qv[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int i = i0 + 8 * u;
+          qv[u] = i < cnt ? *reinterpret_cast<const float4*>(q4 + (size_t)srow[i] * k) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int i = min(i0 + 8 * u, cnt - 1);   // past the end the products are zero
+          const float sh = swh[i], sl = swl[i];
+          const float q[4] = {qv[u].x, qv[u].y, qv[u].z, qv[u].w};
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            const float pp = __fmul_rn(q[v], sh), e = fmaf(q[v], sh, -pp), tt = fmaf(q[v], sl, e);
+            const float uu = __fadd_rn(h[v], pp), bb = __fsub_rn(uu, h[v]);
+            l[v] = __fadd_rn(l[v], __fadd_rn(__fadd_rn(__fsub_rn(h[v], __fsub_rn(uu, bb)), __fsub_rn(pp, bb)), tt));
+            h[v] = uu;
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) res[u] = ds2d(h[u], l[u]);
+  } else if (sizeof(TH) == 4) {
     float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 4
     for (int i = warp; i < cnt; i += 8) {
@@ -252,7 +291,7 @@ __device__ void gram_item(const PersistArgs& A, int a, int it, unsigned char* sm
     for (int u = 0; u < 4; ++u) res[u] = acc[u];
   }
 #pragma unroll
-  for (int u = 0; u < 4; ++u) red[warp][lane + 32 * u] = res[u];
+  for (int u = 0; u < 4; ++u) red[warp][vec ? 4 * lane + u : lane + 32 * u] = res[u];
   __syncthreads();
   if (tid < P_GC) {
     const int cc = ct * P_GC + tid;
@@ -261,13 +300,15 @@ __device__ void gram_item(const PersistArgs& A, int a, int it, unsigned char* sm
     for (int w = 0; w < 8; ++w) v += red[w][tid];
     if (cc < a) A.gram_part[((size_t)ch * a + cc) * k + g] = v;
   }
+  __syncthreads();   // the warps' sums are read before the next tile's
+  }
 }
 
 // P1: the Gram items and the G^T S(r) items as one list (balanced over the CTAs), then Z = S(r)
 template <typename TH, typename TL>
 __device__ void phase_one(const PersistArgs& A, int a, unsigned char* smem) {
   const int n_gtv = A.L.n_G > 0 ? A.L.n_occ * ((A.k + P_GTV_COLS - 1) / P_GTV_COLS) : 0;
-  const int n_gram = a > 0 ? ((a + P_GC - 1) / P_GC) * A.k * A.gs_chunks : 0;
+  const int n_gram = a > 0 ? gram_parts(A, a) * A.k * A.gs_chunks : 0;
   for (int it = blockIdx.x; it < n_gtv + n_gram; it += A.ncta) {
     if (it < n_gtv) gtv_item<TL, true>(A, it, smem);
     else gram_item<TH>(A, a, it - n_gtv, smem);
@@ -437,6 +478,109 @@ __device__ void phase_tall(const PersistArgs& A, int a, unsigned char* smem) {
       for (; q < splits; ++q) v0 += part[(size_t)q * n * k + o];
       const int row = r0 + idx / k, g = idx % k;
       A.Zr[o] = A.Zr[o] - gapply(A, row, g) - to_f64((v0 + v1) + (v2 + v3));
+    }
+  }
+}
+
+// The same for an FP32 history of width K (a multiple of 4): K / 4 lanes hold a row, four history columns each.  A row's
+// K entries of a block are contiguous and so are the rows, so a warp reads whole lines, 16 bytes a lane and eight blocks
+// in flight; the block's coefficients come from shared memory.  Items (row tile, history split).  The phase is
+// bound by the bytes in flight from L2, of which the 64-row form above keeps a fourth.
+template <int K>
+__device__ void phase_tall_rows(const PersistArgs& A, int a, unsigned char* smem) {
+  constexpr int Q = K / 4, ROWS = PT / Q, U = 8;                                            // U blocks in flight
+  constexpr int CB = (P_SMEM - 64) / (4 * K * K) < 32 ? (P_SMEM - 64) / (4 * K * K) : 32;   // blocks staged at once
+  float* sc = reinterpret_cast<float*>(smem);                                               // [block][column][g]
+  int* s_last = reinterpret_cast<int*>(smem + 4 * CB * K * K);
+  const float* Wh = (const float*)A.Wh;
+  float* part = (float*)A.tu_part;
+  const int n = A.n, tid = threadIdx.x, nblk = a / K;
+  const int tiles = (n + ROWS - 1) / ROWS, splits = A.tu_vsplits, per = (nblk + splits - 1) / splits;
+  const int q = tid % Q;
+  for (int it = blockIdx.x; it < tiles * splits; it += A.ncta) {
+    const int tile = it % tiles, sp = it / tiles;
+    const int r0 = tile * ROWS, row = r0 + tid / Q;
+    const bool ok = row < n;
+    const int b0 = min(nblk, sp * per), b1 = min(nblk, b0 + per);
+    const float* w = Wh + (size_t)(ok ? row : 0) * K + 4 * q;
+    float acc[K];
+#pragma unroll
+    for (int g = 0; g < K; ++g) acc[g] = 0.f;
+    for (int c0 = b0; c0 < b1; c0 += CB) {
+      const int cb = min(CB, b1 - c0);
+      __syncthreads();   // the previous coefficients are consumed
+      for (int i = tid; i < cb * K * K; i += PT) sc[i] = from_f64<float>(A.C[(size_t)c0 * K * K + i]);
+      __syncthreads();
+      for (int u0 = 0; u0 < cb; u0 += U) {
+        float4 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          v[u] = u0 + u < cb ? *reinterpret_cast<const float4*>(w + (size_t)(c0 + u0 + u) * n * K)
+                             : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const float* cu = sc + (size_t)min(u0 + u, cb - 1) * K * K + 4 * q * K;
+          const float x[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int g = 0; g < K; g += 4) {
+              const float4 c4 = *reinterpret_cast<const float4*>(cu + e * K + g);
+              acc[g] = fmaf(x[e], c4.x, acc[g]);
+              acc[g + 1] = fmaf(x[e], c4.y, acc[g + 1]);
+              acc[g + 2] = fmaf(x[e], c4.z, acc[g + 2]);
+              acc[g + 3] = fmaf(x[e], c4.w, acc[g + 3]);
+            }
+        }
+      }
+    }
+#pragma unroll
+    for (int g = 0; g < K; ++g)
+#pragma unroll
+      for (int o = 1; o < Q; o <<= 1) acc[g] += __shfl_xor_sync(FULL, acc[g], o);
+    // lane q of the row keeps columns 4 q .. 4 q + 3
+    float4 mine = make_float4(acc[0], acc[1], acc[2], acc[3]);
+#pragma unroll
+    for (int p = 1; p < Q; ++p)
+      if (q == p) mine = make_float4(acc[4 * p], acc[4 * p + 1], acc[4 * p + 2], acc[4 * p + 3]);
+    if (splits == 1) {
+      if (ok) {
+        const float m4[4] = {mine.x, mine.y, mine.z, mine.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const size_t o = (size_t)row * K + 4 * q + e;
+          A.Zr[o] = A.Zr[o] - gapply(A, row, 4 * q + e) - to_f64(m4[e]);
+        }
+      }
+      continue;
+    }
+    if (ok) *reinterpret_cast<float4*>(part + ((size_t)sp * n + row) * K + 4 * q) = mine;
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+      const unsigned prev = atomicAdd(&A.tu_tickets[tile], 1u);
+      *s_last = prev == (unsigned)splits - 1;
+      if (*s_last) A.tu_tickets[tile] = 0u;
+    }
+    __syncthreads();
+    const bool last = *s_last;
+    __syncthreads();   // read before the next item's coefficients or flag
+    if (!last) continue;
+    __threadfence();
+    // the last CTA of the tile: one element per thread, its splits on four running sums
+    const int rows = min(ROWS, n - r0);
+    for (int idx = tid; idx < rows * K; idx += PT) {
+      const size_t o = (size_t)r0 * K + idx;
+      float v0 = 0.f, v1 = 0.f, v2 = 0.f, v3 = 0.f;
+      int p = 0;
+      for (; p + 3 < splits; p += 4) {
+        v0 += part[(size_t)p * n * K + o];
+        v1 += part[(size_t)(p + 1) * n * K + o];
+        v2 += part[(size_t)(p + 2) * n * K + o];
+        v3 += part[(size_t)(p + 3) * n * K + o];
+      }
+      for (; p < splits; ++p) v0 += part[(size_t)p * n * K + o];
+      A.Zr[o] = A.Zr[o] - gapply(A, r0 + idx / K, idx % K) - to_f64((v0 + v1) + (v2 + v3));
     }
   }
 }
@@ -744,7 +888,13 @@ __global__ void __launch_bounds__(PT) k_persist(PersistArgs A) {
     }
     if (A.L.n_G > 0) phase_small_gemm(A);
     if (!phase_end(1)) return;
-    phase_tall<TH, KP>(A, a, smem);   // P3
+    // P3
+    if (sizeof(TH) == 4 && A.tu_vsplits > 0 && a > 0) {
+      if (KP == 8 && A.k == 4) phase_tall_rows<4>(A, a, smem);
+      else phase_tall_rows<KP>(A, a, smem);
+    } else {
+      phase_tall<TH, KP>(A, a, smem);
+    }
     if (!phase_end(2)) return;
     phase_local<TL>(A, smem);         // P4 + P5: gather fused into the local products
     if (!phase_end(4)) return;
