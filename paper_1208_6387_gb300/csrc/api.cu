@@ -1241,7 +1241,7 @@ void build_structure(fetirp_ctx ctx, int64_t n_lambda, const double* c_host, con
   else ctx->c.zero(s);
   ctx->Xc.ensure((size_t)std::max(ctx->n_G, 1) * 64);
   ctx->Ac.ensure((size_t)std::max(ctx->n_G, 1) * 64);
-  ctx->sg_part.ensure((size_t)small_gemm_parts(std::max(ctx->n_G, 1)) * std::max(ctx->n_G, 1) * 64);
+  ctx->sg_part.ensure((size_t)SMALL_GEMM_MAX_PARTS * std::max(ctx->n_G, 1) * 64);
   if (ctx->n_G > 0) {
     gtg_dense(L, nullptr, nullptr, ctx->n_pairs, ctx->d_pair_s.p, ctx->d_pair_t.p, ctx->GtG.p, s);
     ctx->planG = dense_plan(ctx->n_Gpad / TILE);

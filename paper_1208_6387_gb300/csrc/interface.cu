@@ -676,6 +676,8 @@ void gt_v_ds(const Layout& L, const double* V, int k, double* X, cudaStream_t s)
   const int max_links = L.gtv_chunk * L.gtv_chunks;   // >= the links of the largest occurrence
   int nch = L.gtv_chunks;
   if (8 * 4 * workers > L.gtv_chunk) nch = std::max(1, std::min(nch, ceil_div(max_links, 8 * 4 * workers)));
+  // but CTAs for every SM come first (27 occurrences, k = 9: 108 CTAs took 31 us)
+  nch = std::max(nch, std::min(L.gtv_chunks, ceil_div(2 * 152, L.n_occ)));
   const int chunk = (int)round_up(ceil_div(max_links, nch), 32);
   const dim3 grid(L.n_occ, ceil_div(max_links, chunk));
   if (k > 32) k_gt_v_ds<32, true><<<grid, GTV_THREADS, 0, s>>>(L, V, k, X, chunk);

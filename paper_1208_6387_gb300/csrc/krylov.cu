@@ -530,7 +530,9 @@ template void gram<double, double>(int, int, int, const double*, int, const doub
                                    DBuf<double>&, cudaStream_t);
 
 // up to four chunks per SM (the sums are FP64-pipe bound: more resident warps keep the pipe busy)
-int eta_chunks(int n) { return std::max(1, std::min(608, ceil_div(n, 256))); }
+// Row chunks of the eta products: 64 rows each (two staging steps) until there are four CTAs per SM.  With 256 rows a
+// structure of 14,049 rows ran 55 CTAs (k = 9: 42 us; so 16).
+int eta_chunks(int n) { return std::max(1, std::min(608, ceil_div(n, 64))); }
 
 // (h, l) += (bh, bl) for unevaluated FP32 pairs: Knuth's TwoSum of the high parts, the low parts and the error
 // added, then renormalised (Dekker's Fast2Sum)
@@ -680,6 +682,11 @@ int small_gemm_parts(int m) {
   return std::max(1, std::min(SMALL_GEMM_MAX_PARTS, std::min(ceil_div(608, ceil_div(m, 4)), m / 128)));
 }
 
+// The double-single form has no FP64 rate to fill but a long dependent chain per term: slices of >= 32 terms
+static int small_gemm_ds_parts(int m) {
+  return std::max(1, std::min(SMALL_GEMM_MAX_PARTS, std::min(ceil_div(608, ceil_div(m, 4)), m / 32)));
+}
+
 void small_gemm(int m, int k, const double* A, const double* B, double* C, cudaStream_t s, double* part) {
   if (m <= 0 || k <= 0) return;
   if (k > 64) throw Error(1, "k > 64");
@@ -734,7 +741,7 @@ void small_gemm_ds(int m, int k, const float* Ah, const float* Al, const float* 
                    cudaStream_t s, double* part) {
   if (m <= 0 || k <= 0) return;
   if (k > 64) throw Error(1, "k > 64");
-  const int parts = part ? small_gemm_parts(m) : 1;
+  const int parts = part ? small_gemm_ds_parts(m) : 1;
   k_small_gemm_ds<<<dim3(ceil_div(m, 4), parts), 128, 0, s>>>(m, k, Ah, Al, Bh, Bl, parts > 1 ? part : C);
   FETIRP_LAUNCH_CHECK();
   if (parts > 1) {
