@@ -480,7 +480,7 @@ void factor_stage_a(PatternData& P, double pivot_tol, const CholAux& aux, cudaSt
   P.diag0.ensure(npad);
   P.zp.ensure(npad);
   copy_diag(P.L.p, npad, P.diag0.p, s);
-  chol_tiles(P.L.p, npad, P.plan, P.diag0.p, P.zp.p, pivot_tol, s, &aux);
+  chol_tiles(P.L.p, n, npad, P.plan, P.diag0.p, P.zp.p, pivot_tol, s, &aux);
   P.Dinv.ensure((size_t)npad * TILE);
   tile_inverses(P.L.p, npad, P.zp.p, P.Dinv.p, s);
   P.h_zp.resize(npad);
@@ -775,7 +775,7 @@ void spd_inverse(fetirp_ctx ctx, const double* A_rowmajor, int n, int npad, Tile
   }
   zp.ensure(npad);
   copy_diag(A.p, npad, diag.p, s);
-  chol_tiles(A.p, npad, plan, diag.p, zp.p, 1e-13, s);
+  chol_tiles(A.p, n, npad, plan, diag.p, zp.p, 1e-13, s);
   std::vector<int> h(npad);
   FETIRP_CUDA(cudaMemcpyAsync(h.data(), zp.p, sizeof(int) * npad, cudaMemcpyDeviceToHost, s));
   FETIRP_CUDA(cudaStreamSynchronize(s));
@@ -2071,6 +2071,11 @@ PersistArgs persist_args(fetirp_ctx ctx, bool fp64, TH* Wh, TH* Qh) {
     tiles += A.tiles_m[p] * ceil_div(A.n_rhs[p], 16);
   }
   A.tile_off[n_pat] = tiles;
+  // no more CTAs than the phases have work for: the barriers and the reductions over CTAs are what a small structure
+  // waits for
+  const long long items[4] = {ceil_div(nl, 8), tiles, (long long)L.n_occ * ceil_div(k, 8),
+                              (long long)ceil_div(ctx->hist_cap, 128) * k * ceil_div(ctx->max_group_rows, 128)};
+  A.ncta = (int)std::min<long long>(A.ncta, std::max<long long>(8, *std::max_element(items, items + 4)));
   if (fp64) {
     ctx->Y64.ensure(total); ctx->Z64.ensure(total);
     A.Ybuf = ctx->Y64.p; A.Zbuf = ctx->Z64.p;

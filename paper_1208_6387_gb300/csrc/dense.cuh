@@ -36,7 +36,8 @@ struct CholAux {
   cudaStream_t stream;
   cudaEvent_t panel, rest;
 };
-void chol_tiles(double* A, int npad, const TilePlan& plan, const double* diag0, int* zp, double tol,
+// n: rows of the matrix proper; rows n .. npad - 1 of A are the identity.
+void chol_tiles(double* A, int n, int npad, const TilePlan& plan, const double* diag0, int* zp, double tol,
                 cudaStream_t s, const CholAux* aux = nullptr);
 
 // X <- L^{-1} X (trans = false) or X <- L^{-T} X (trans = true), X column-major npad x nrhs (ld = ldx),

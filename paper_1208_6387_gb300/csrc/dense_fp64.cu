@@ -64,10 +64,11 @@ __global__ void k_zero_zp_rows(double* A, int npad, const int* zp) {
 // column, a_rc -= l_r a_cj, and every column is scaled by 1 / sqrt(d_j) once at the end, in parallel, giving
 // L = L_unit D^{1/2}.  One step of lookahead: thread 0 updates the next diagonal entry first and forms its
 // reciprocal while the other threads finish the update.  Zero pivots (d_j <= tol * diag0_j, or not finite) get
-// a zero multiplier column (no update) and a zero column of L.  The step's column is copied beside the tile, so that a
+// a zero multiplier column (no update) and a zero column of L.  nv: the tile's rows of the matrix; the padding after them
+// is the identity and takes no steps.  The step's column is copied beside the tile, so that a
 // thread's loads of four entries do not wait for its stores, and a thread takes four entries at a time.
 __global__ void __launch_bounds__(256) k_potrf_tile(double* A, int npad, int k, const double* diag0, int* zp,
-                                                    double tol) {
+                                                    double tol, int nv) {
   __shared__ double a[TILE][TILE + 1];   // a[row][col]
   __shared__ double thr[TILE];           // tol * diag0 of the tile's dofs
   __shared__ double dd[TILE];            // pivots d_j (0 for zero pivots), then 1 / sqrt(d_j)
@@ -81,6 +82,7 @@ __global__ void __launch_bounds__(256) k_potrf_tile(double* A, int npad, int k, 
     a[r][c] = T[(size_t)c * npad + r];
   }
   if (tid < TILE) thr[tid] = tol * diag0[k * TILE + tid];
+  if (tid >= nv && tid < TILE) dd[tid] = 1.0;
   __syncthreads();
   if (tid == 0) {
     const double d = a[0][0];
@@ -90,7 +92,7 @@ __global__ void __launch_bounds__(256) k_potrf_tile(double* A, int npad, int k, 
   }
   __syncthreads();
   const int rr = tid % TILE, cg = tid / TILE;   // update: row rr, columns j+1+cg, j+5+cg, ...
-  for (int j = 0; j + 1 < TILE; ++j) {
+  for (int j = 0; j + 1 < nv; ++j) {
     const double rinv = s_rinv;
     if (tid > j && tid < TILE) {
       const double v = a[tid][j];
@@ -552,13 +554,13 @@ void zero_zp_rows(double* A, int npad, const int* zp, cudaStream_t s) {
   FETIRP_LAUNCH_CHECK();
 }
 
-void chol_tiles(double* A, int npad, const TilePlan& plan, const double* diag0, int* zp, double tol,
+void chol_tiles(double* A, int n, int npad, const TilePlan& plan, const double* diag0, int* zp, double tol,
                 cudaStream_t s, const CholAux* aux) {
   // With aux, a step's update is split: the next column's tiles on s, so that its factorisation and panel solve (the
   // serial chain of the algorithm) go on, and the rest on aux beside them, in the same order for every tile.
   bool pending = false;   // aux holds updates that s has not waited for
   for (int k = 0; k < plan.nt; ++k) {
-    k_potrf_tile<<<1, 256, 0, s>>>(A, npad, k, diag0, zp, tol);
+    k_potrf_tile<<<1, 256, 0, s>>>(A, npad, k, diag0, zp, tol, std::min(TILE, n - k * TILE));
     FETIRP_LAUNCH_CHECK();
     const int nr = plan.col_off[k + 1] - plan.col_off[k];
     if (nr == 0) continue;
