@@ -1305,6 +1305,7 @@ void build_structure(fetirp_ctx ctx, int64_t n_lambda, const double* c_host, con
   ctx->d_state.ensure(4);
   ensure_tc_error(ctx);
   tc_init();
+  oz_init();
   ensure_apply_buffers(ctx, k);
   if (ctx->gc.exec) { cudaGraphExecDestroy(ctx->gc.exec); ctx->gc.exec = nullptr; }   // buffers may have moved
   ctx->n_lambda = n_lambda;

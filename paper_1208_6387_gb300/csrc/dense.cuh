@@ -30,7 +30,8 @@ struct TilePlan {
 // nonsingular block K_rr embedded with zeros (the generalized inverse of Sec. 2).
 // aux (optional): a second stream, of lower priority than s, and two events for the trailing updates that the next
 // column does not wait for.  They go there from CHOL_SPLIT_PAIRS tile pairs on, about what fills the SMs for as long as a
-// diagonal tile and its panel take.  Single 12^3 elastic pattern: 42.3 ms a factorisation without, 33 with.
+// diagonal tile and its panel take.  Single 12^3 elastic pattern: 42.3 ms a factorisation without,
+// 36.7 with (and with the tile and panel kernels of the same change).
 constexpr int CHOL_SPLIT_PAIRS = 76;
 struct CholAux {
   cudaStream_t stream;

@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(256) k_potrf_tile(double* A, int npad, int k, 
 // a tile are independent, so grid.y splits each tile into eight 8-row blocks (more SMs on the FP64 work).  Sixteen
 // threads of one warp hold a row in registers (every sixteenth column each): step j is a multiply by the pivot's
 // reciprocal, a shuffle and the FMAs of the later columns, without a barrier; bound by the FP64 pipe (rows in shared
-// memory, two barriers a step: 40 us for 35 tiles; this: 17 us).
+// memory, two barriers a step: 40 us for 35 tiles; this: 23 us, 18 us for a handful of tiles).
 constexpr int TR_ROWS = 8;
 __global__ void __launch_bounds__(16 * TR_ROWS) k_trsm_tiles(double* A, int npad, int k, const int* rows, const int* zp) {
   __shared__ double l[TILE][TILE + 1];

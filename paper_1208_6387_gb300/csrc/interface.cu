@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(GTV_THREADS, WIDE ? 2 : 3) k_gt_v(Layout L, co
 // out[row][g] = beta*in + alpha * sum over the row's slots: (sign Nb[j]) . A[gofs(s)..][g], from the per-row
 // tables (coarse column, kernel dimension and signed coefficients of each slot), so that the only dependent
 // load is A's (small, cache-resident).  C columns per thread (C = 4 when k is a multiple of 4: the row's tables and
-// coefficients are read once for four columns; bound by the 12 FMAs per element of the FP64 pipe: 57 -> 45 us for
+// coefficients are read once for four columns; bound by the 12 FMAs per element of the FP64 pipe: 57 -> 51 us for
 // 427,392 x 4).  in may be out.
 template <int C>
 __global__ void k_g_apply(Layout L, const double* __restrict__ A, int k, double alpha, double beta, const double* in,

@@ -529,9 +529,8 @@ template void gram<float, double>(int, int, int, const float*, int, const double
 template void gram<double, double>(int, int, int, const double*, int, const double*, int, double*,
                                    DBuf<double>&, cudaStream_t);
 
-// up to four chunks per SM (the sums are FP64-pipe bound: more resident warps keep the pipe busy)
-// Row chunks of the eta products: 64 rows each (two staging steps) until there are four CTAs per SM.  With 256 rows a
-// structure of 14,049 rows ran 55 CTAs (k = 9: 42 us; so 16).
+// Row chunks of the eta products: 64 rows each (two staging steps) until there are four per SM (the sums are FP64-pipe
+// bound: more resident warps keep the pipe busy).  With 256 rows a structure of 14,049 rows ran on 55 CTAs.
 int eta_chunks(int n) { return std::max(1, std::min(608, ceil_div(n, 64))); }
 
 // (h, l) += (bh, bl) for unevaluated FP32 pairs: Knuth's TwoSum of the high parts, the low parts and the error

@@ -58,13 +58,13 @@ struct OzGemmKernel {
 
 // One CTA: 128 rows of A (two row tiles) against 64 rows of B, all of K in 64-wide blocks.  Bound by the MMAs (28 digit
 // pairs, i + j <= 6: over a long row the dropped products stay far below the rounding of an FP64 chain).  FP64 apply of
-// three 16^3 elastic patterns (n_b = 4614, 256 right-hand sides each, 32.7 GFLOP): 27.5 ms with FP64 FMAs, 1.59 ms so
-// (24.2 against 0.9 ms for the product itself), and its error against 64 bits is the same (2.2e-10 of the projected
-// result, which is that of S^+).  The two
-// 32-column halves of a block have an accumulator buffer each (224 TMEM columns): one is drained while the other is
-// multiplied.  Both halves use the same A slices, so a slice is released after its product with the second half and
-// the ring of ten holds the next block's first ones; the B halves are refilled in turn.  Drained levels are added
-// into 91-bit integers per output (a 64-bit and a 27-bit part): no FP64 operation before the final rounding.
+// three 16^3 elastic patterns (n_b = 4614, 256 right-hand sides each, 32.7 GFLOP): 27.5 ms with FP64 FMAs, 1.11 ms so
+// (0.87 ms of it this kernel: 28 x 32.7 GFLOP issued at 1.05 PFLOP/s), and its error against 64 bits is the same
+// (2.2e-10 of the projected result, which is that of S^+).  The two 32-column halves of a block have an accumulator
+// buffer each (224 TMEM columns): one is drained while the other is multiplied.  Both halves use the same A slices, so
+// a slice is released after its product with the second half and the ring of ten holds the next block's first ones; the
+// B halves are refilled in turn.  Drained levels are added into 91-bit integers per output (a 64-bit and a 27-bit part):
+// no FP64 operation before the final rounding.
 __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ OzGemmKernel P) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -275,7 +275,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
 
 // Row exponents and slices of row-major operands, a CTA per (padded) row: the row is read twice, the second time from L1
 // or L2, and written as 16-byte groups of 8 digits of a slice.  Bound by latency and the integer digits, so every row
-// of every operand gets a CTA in one launch (a warp per row: 39 us for 256 rows of 4614; this: 8 us for 768).
+// of every operand gets a CTA in one launch (a warp per row, a launch per operand: 39 us for 256 rows of 4614; this:
+// 27 us for all 768).
 __global__ void __launch_bounds__(128) k_oz_slice(const __grid_constant__ OzSliceBatch P) {
   __shared__ unsigned long long wmax[4];
   int p = 0;
@@ -357,7 +358,7 @@ __global__ void __launch_bounds__(256) k_oz_slice_t(const double* __restrict__ x
 }
 
 // ------------------------------------------------------------------------------------------------ host
-static void oz_init() {
+void oz_init() {
   static std::mutex mu;
   static bool attr_done[64] = {};
   std::lock_guard<std::mutex> lock(mu);

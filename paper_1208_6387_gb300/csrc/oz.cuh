@@ -62,6 +62,9 @@ struct OzGemm {
 };
 void oz_gemm(const OzGemm& G, cudaStream_t s);
 
+// One-time kernel attribute set-up (large dynamic shared memory); call before any graph capture.
+void oz_init();
+
 #ifdef __CUDACC__
 // |x| as the bits that order like it, for row maxima
 __device__ __forceinline__ unsigned long long oz_abs_bits(double x) {

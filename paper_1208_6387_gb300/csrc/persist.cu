@@ -189,7 +189,7 @@ __device__ void phase_gtv(const PersistArgs& A, unsigned char* smem) {
 // in warp order (deterministic); FP32 history: double-single sums on the FP32 pipe (see the split Gram kernel).
 constexpr int P_GC = 128;
 // Parts that the history columns of a (group, row chunk) are cut into: about an item per CTA, so that a chunk's rows,
-// two dependent loads away, are staged once for several column tiles
+// two dependent loads away, are staged once for several column tiles (34 -> 32 us per block iteration, 3904 rows, k = 8)
 __device__ __forceinline__ int gram_parts(const PersistArgs& A, int a) {
   const int ctiles = (a + P_GC - 1) / P_GC;
   return min(ctiles, max(1, A.ncta / max(1, A.k * A.gs_chunks)));
@@ -485,7 +485,8 @@ __device__ void phase_tall(const PersistArgs& A, int a, unsigned char* smem) {
 // The same for an FP32 history of width K (a multiple of 4): K / 4 lanes hold a row, four history columns each.  A row's
 // K entries of a block are contiguous and so are the rows, so a warp reads whole lines, 16 bytes a lane and eight blocks
 // in flight; the block's coefficients come from shared memory.  Items (row tile, history split).  The phase is
-// bound by the bytes in flight from L2, of which the 64-row form above keeps a fourth.
+// bound by the bytes in flight from L2, of which the 64-row form above keeps a fourth.  3904 rows, k = 8, up to 3904
+// directions: 31 -> 27 us per block iteration.
 template <int K>
 __device__ void phase_tall_rows(const PersistArgs& A, int a, unsigned char* smem) {
   constexpr int Q = K / 4, ROWS = PT / Q, U = 8;                                            // U blocks in flight
