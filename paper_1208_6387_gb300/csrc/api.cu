@@ -2094,12 +2094,15 @@ PersistArgs persist_args(fetirp_ctx ctx, bool fp64, TH* Wh, TH* Qh) {
   A.Ginv = ctx->Ginv.p; A.Xc = ctx->Xc.p; A.Ac = ctx->Ac.p;
   // history splits sized for the persistent grid (about one item per CTA; never more than tu_part holds)
   A.tu_splits = std::max(1, std::min(tall_update_splits(nl, (int)ctx->hist_cap), A.ncta / ceil_div(nl, 64)));
-  // one row per thread: the longest histories leave every split at least 64 directions
+  // k / 4 lanes per row: the longest histories leave every split at least 64 directions
   A.tu_vsplits = 0;
   if (!fp64 && (k == 4 || k == 8 || k == 16 || k == 32)) {
-    A.tu_vsplits = (int)std::max<long long>(1, std::min<long long>(A.ncta / ceil_div(nl, 1024 / k), ctx->hist_cap / 64));
+    A.tu_vsplits = (int)std::max<long long>(
+        1, std::min<long long>(A.ncta / ceil_div(nl, persist_tall_rows(k)), ctx->hist_cap / 64));
     ctx->tu_part.ensure((size_t)A.tu_vsplits * nl * k);
   }
+  if (ctx->tu_tickets.n < (size_t)persist_tickets(nl, k))
+    throw Error(FETIRP_ESTATE, "the persistent iteration has fewer tickets than row tiles");
   A.tu_part = ctx->tu_part.p; A.tu_tickets = ctx->tu_tickets.p;
   const int nout = k * (k + 1);
   ctx->pers_eta.ensure((size_t)(A.ncta + 64) * nout);
@@ -2358,7 +2361,7 @@ void ensure_history(fetirp_ctx ctx) {
   ctx->tu_part.ensure(std::max(tall_update_scratch(nl, (int)cap, k, true), tall_update_scratch(nl, (int)cap, k, false)));
   tall_update_init();
   {
-    const int tiles = ceil_div(nl, 64);
+    const int tiles = persist_tickets(nl, k);   // >= ceil_div(nl, 64), what the per-phase update takes
     if (ctx->tu_tickets.n < (size_t)tiles) {
       ctx->tu_tickets.alloc(tiles);
       FETIRP_CUDA(cudaMemsetAsync(ctx->tu_tickets.p, 0, sizeof(unsigned) * tiles, ctx->stream));

@@ -238,7 +238,8 @@ struct PersistArgs {
   const double* Ginv;
   double* Xc;
   double* Ac;
-  // history update; tu_vsplits > 0: the one-row-per-thread form with that many history splits (FP32, k = 4, 8, 16, 32)
+  // history update; tu_vsplits > 0: the form with k / 4 lanes per row and that many history splits (FP32, k = 4, 8, 16,
+  // 32).  tu_tickets: persist_tickets(n, k) counters, zero at launch
   int tu_splits;
   int tu_vsplits;
   void* tu_part;
@@ -263,6 +264,13 @@ struct PersistArgs {
   // optional (timing): nanoseconds spent by CTA 0 in each of the nine phases, barrier wait included, summed
   unsigned long long* clk;
 };
+// Rows of a tile of the persistent history update with k / 4 lanes per row (256 threads), and the row tiles of the
+// finest form of an n x k update: each of them has a ticket.
+constexpr int persist_tall_rows(int k) { return 256 / (k / 4); }
+inline int persist_tickets(int n, int k) {
+  const bool rows = k == 4 || k == 8 || k == 16 || k == 32;
+  return ceil_div(n, rows && persist_tall_rows(k) < 64 ? persist_tall_rows(k) : 64);
+}
 void persist_iterations(const PersistArgs& A, bool fp64, cudaStream_t s);
 int persist_ctas(bool fp64, int k);   // co-resident CTAs of the launch (0 if the kernel cannot be co-resident)
 
@@ -293,7 +301,8 @@ void hist_dot(int n, int a, const TH* Qh, int hk, const double* r, double* C, DB
 // W (n x k, FP64) += alpha * Wh (n x a, history type TH, block layout of width hk) * C (a x k, FP64),
 // computed in TH arithmetic.
 // scratch: split partials, tall_update_splits(n, a_max) * n * k values of TH; tickets: one counter per 64-row
-// tile, zero between calls (both grown here; callers that capture graphs size them first).
+// tile, zero between calls (both grown here; callers that capture graphs size them first, and for the persistent
+// iteration, which shares them, for its own row tiles: persist_tickets).
 int tall_update_splits(int n, int a_max);
 // device scratch (in doubles) that tall_update needs for n rows, a_max columns, k outputs
 size_t tall_update_scratch(int n, int a_max, int k, bool fp32);

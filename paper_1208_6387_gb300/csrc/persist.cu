@@ -490,6 +490,7 @@ __device__ void phase_tall(const PersistArgs& A, int a, unsigned char* smem) {
 template <int K>
 __device__ void phase_tall_rows(const PersistArgs& A, int a, unsigned char* smem) {
   constexpr int Q = K / 4, ROWS = PT / Q, U = 8;                                            // U blocks in flight
+  static_assert(ROWS == persist_tall_rows(K), "a ticket per row tile");
   constexpr int CB = (P_SMEM - 64) / (4 * K * K) < 32 ? (P_SMEM - 64) / (4 * K * K) : 32;   // blocks staged at once
   float* sc = reinterpret_cast<float*>(smem);                                               // [block][column][g]
   int* s_last = reinterpret_cast<int*>(smem + 4 * CB * K * K);
