@@ -2,6 +2,7 @@
 // subdomains), right-looking multi-right-hand-side triangular solves and a strided generic GEMM.
 #include <algorithm>
 
+#include "chol_schedule.cuh"
 #include "dense.cuh"
 
 namespace fetirp {
@@ -556,40 +557,36 @@ void zero_zp_rows(double* A, int npad, const int* zp, cudaStream_t s) {
 
 void chol_tiles(double* A, int n, int npad, const TilePlan& plan, const double* diag0, int* zp, double tol,
                 cudaStream_t s, const CholAux* aux) {
-  // With aux, a step's update is split: the next column's tiles on s, so that its factorisation and panel solve (the
-  // serial chain of the algorithm) go on, and the rest on aux beside them, in the same order for every tile.
-  bool pending = false;   // aux holds updates that s has not waited for
-  for (int k = 0; k < plan.nt; ++k) {
-    k_potrf_tile<<<1, 256, 0, s>>>(A, npad, k, diag0, zp, tol, std::min(TILE, n - k * TILE));
-    FETIRP_LAUNCH_CHECK();
-    const int nr = plan.col_off[k + 1] - plan.col_off[k];
-    if (nr == 0) continue;
-    const int* rows = plan.d_col_rows.p + plan.col_off[k];
-    k_trsm_tiles<<<dim3(nr, TILE / TR_ROWS), 16 * TR_ROWS, 0, s>>>(A, npad, k, rows, zp);
-    FETIRP_LAUNCH_CHECK();
-    const int2* pairs = plan.d_pairs.p + plan.pair_off[k];
-    const int np = plan.pair_off[k + 1] - plan.pair_off[k];
-    const int first = plan.col_rows[plan.col_off[k]] == k + 1 ? nr : 0;   // pairs of column k + 1
-    const bool split = aux && np - first >= CHOL_SPLIT_PAIRS;
-    if (split) FETIRP_CUDA(cudaEventRecord(aux->panel, s));
-    if (pending) {   // every earlier update of these tiles
-      FETIRP_CUDA(cudaStreamWaitEvent(s, aux->rest, 0));
-      pending = false;
-    }
-    const int on_s = split ? first : np;
-    if (on_s > 0) {
-      k_update_pairs<<<dim3(on_s, 4), 256, 0, s>>>(A, npad, k, pairs);
+  struct {
+    double* A;
+    int n, npad;
+    const TilePlan& plan;
+    const double* diag0;
+    int* zp;
+    double tol;
+    cudaStream_t s;
+    const CholAux* aux;
+    void tile(int k) {
+      k_potrf_tile<<<1, 256, 0, s>>>(A, npad, k, diag0, zp, tol, std::min(TILE, n - k * TILE));
       FETIRP_LAUNCH_CHECK();
     }
-    if (split) {
+    void panel(int k) {
+      const int nr = plan.col_off[k + 1] - plan.col_off[k];
+      k_trsm_tiles<<<dim3(nr, TILE / TR_ROWS), 16 * TR_ROWS, 0, s>>>(A, npad, k, plan.d_col_rows.p + plan.col_off[k], zp);
+      FETIRP_LAUNCH_CHECK();
+    }
+    void update(int k, int p0, int count, bool side) {
+      k_update_pairs<<<dim3(count, 4), 256, 0, side ? aux->stream : s>>>(A, npad, k, plan.d_pairs.p + p0);
+      FETIRP_LAUNCH_CHECK();
+    }
+    void fork() {
+      FETIRP_CUDA(cudaEventRecord(aux->panel, s));
       FETIRP_CUDA(cudaStreamWaitEvent(aux->stream, aux->panel, 0));
-      k_update_pairs<<<dim3(np - first, 4), 256, 0, aux->stream>>>(A, npad, k, pairs + first);
-      FETIRP_LAUNCH_CHECK();
-      FETIRP_CUDA(cudaEventRecord(aux->rest, aux->stream));
-      pending = true;
     }
-  }
-  if (pending) FETIRP_CUDA(cudaStreamWaitEvent(s, aux->rest, 0));
+    void mark() { FETIRP_CUDA(cudaEventRecord(aux->rest, aux->stream)); }
+    void join() { FETIRP_CUDA(cudaStreamWaitEvent(s, aux->rest, 0)); }
+  } ops{A, n, npad, plan, diag0, zp, tol, s, aux};
+  chol_schedule(plan.nt, plan.col_off.data(), plan.col_rows.data(), plan.pair_off.data(), aux ? CHOL_SPLIT_PAIRS : 0, ops);
   zero_zp_rows(A, npad, zp, s);
 }
 
