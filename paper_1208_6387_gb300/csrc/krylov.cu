@@ -608,17 +608,14 @@ __global__ void k_eta_group_sums(int nout, int chunks, const double* __restrict_
 
 int eta_partials(int n, int k, const double* W, const double* Q, const double* r, DBuf<double>& partial,
                  cudaStream_t s, bool ds, int* n_read) {
-  const bool small = ds && k <= 4;
-  // narrow blocks: one CTA per SM, a few thousand rows each (every thread sums several rows before the
-  // per-CTA reduction); otherwise up to 608 chunks of >= 256 rows
+  // k = 4: one CTA per SM, a few thousand rows each (every thread sums several rows before the per-CTA reduction, its
+  // pairs added over the warp); otherwise up to 608 chunks of >= 64 rows, whose threads' sums are added in FP64
+  const bool small = ds && k == 4;
   const int chunks = small ? std::max(1, std::min(152, ceil_div(n, 1024))) : eta_chunks(n);
   const int rows = ceil_div(n, chunks);
   const int nout = k * (k + 1);
   partial.ensure((size_t)(chunks + ETA_GROUPS) * nout);
-  if (small && k == 4) k_eta_small_ds<4><<<chunks, 256, 0, s>>>(n, W, Q, r, rows, partial.p);
-  else if (small && k == 3) k_eta_small_ds<3><<<chunks, 256, 0, s>>>(n, W, Q, r, rows, partial.p);
-  else if (small && k == 2) k_eta_small_ds<2><<<chunks, 256, 0, s>>>(n, W, Q, r, rows, partial.p);
-  else if (small) k_eta_small_ds<1><<<chunks, 256, 0, s>>>(n, W, Q, r, rows, partial.p);
+  if (small) k_eta_small_ds<4><<<chunks, 256, 0, s>>>(n, W, Q, r, rows, partial.p);
   else if (ds) k_eta_partial_ds<<<chunks, 256, 0, s>>>(n, k, W, Q, r, rows, partial.p);
   else k_eta_partial<<<chunks, 256, 0, s>>>(n, k, W, Q, r, rows, partial.p);
   FETIRP_LAUNCH_CHECK();

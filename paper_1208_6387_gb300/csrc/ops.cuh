@@ -312,7 +312,7 @@ template <typename TH>
 void tall_update(int n, int a_max, const int* d_a, int k, const TH* Wh, int hk, const double* C, double alpha,
                  double* W, DBuf<double>& scratch, DBuf<unsigned>& tickets, cudaStream_t s);
 // Row-chunk partials of [eta | wr] = W^T [Q | r], a k x (k+1) block, FP64 sums: at most eta_chunks(n) of them
-// (k <= 4 with ds: one per SM).  With more than ETA_GROUPS chunks they are first added into ETA_GROUPS group sums
+// (k = 4 with ds: one per SM).  With more than ETA_GROUPS chunks they are first added into ETA_GROUPS group sums
 // (fixed order) stored after the chunks.  The return value is the offset, in blocks of k (k+1), of what
 // normalise() must add, and *n_read their number (the chunks themselves, or the ETA_GROUPS group sums).
 constexpr int ETA_GROUPS = 16;
