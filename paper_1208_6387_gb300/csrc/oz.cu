@@ -10,8 +10,8 @@ namespace fetirp {
 namespace {
 
 constexpr int THREADS = 320;                         // producer warp, MMA warp, 8 epilogue warps
-constexpr int EPI_WARPS = 8;
-constexpr int BUF_COLS = 256;                        // TMEM columns between the two accumulator buffers (7 x 32 used)
+constexpr int EPI_WARPS = 8, EPI_COLS = OZ_COLS / (EPI_WARPS / 4);   // a warp's columns of its 32 rows
+constexpr int TMEM_COLS = 512;                       // 7 levels of 64 used
 
 // K-major operand, 128-byte swizzle, 8-row groups 1024 bytes apart
 __device__ __forceinline__ uint64_t desc128(const void* p) {
@@ -46,9 +46,11 @@ __device__ __forceinline__ double rounded(long long hi, long long lo, int w, int
   return scaled_i64((hi << room) + (lo >> (w - room)), e - room);
 }
 
-constexpr int G_RING = 10;                              // A slices (128 rows, 16 KB) in flight
-constexpr int G_SLICE = 4 * OZ_SLICE_HALF;
-constexpr int G_SMEM = G_RING * G_SLICE + OZ_TILE + 1024 + 512;
+constexpr int G_A = 2 * OZ_SLICE;                       // an A slice of 128 rows: 16 KB
+constexpr int G_ZEROS = OZ_PAD * OZ_SLICE;              // zero slices in front of B
+constexpr int G_B = G_ZEROS + OZ_TILE;
+constexpr int G_SMEM = OZ_RING * G_A + G_B + 1024 + 512;
+static_assert(G_SMEM <= 227 * 1024, "shared memory of a CTA");
 
 struct OzGemmKernel {
   OzGemm G;
@@ -56,33 +58,27 @@ struct OzGemmKernel {
 };
 }  // namespace
 
-// One CTA: 128 rows of A (two row tiles) against 64 rows of B, all of K in 64-wide blocks.  Bound by the MMAs' rate (28
-// digit pairs, i + j <= 6: over a long row the dropped products stay far below the rounding of an FP64 chain).  FP64 apply of
-// three 16^3 elastic patterns (n_b = 4614, 256 right-hand sides each, 32.7 GFLOP): 27.5 ms with FP64 FMAs, 1.11 ms so
-// (0.87 ms of it this kernel: 28 x 32.7 GFLOP issued at 1.05 PFLOP/s), and its error against 64 bits is the same
-// (2.2e-10 of the projected result, which is that of S^+).  The two 32-column halves of a block have an accumulator
-// buffer each (224 TMEM columns): one is drained while the other is multiplied.  Both halves use the same A slices, so
-// a slice is released after its product with the second half and the ring of ten holds the next block's first ones; the
-// B halves are refilled in turn.  Drained levels are added into 91-bit integers per output (a 64-bit and a 27-bit part):
-// no FP64 operation before the final rounding.  The tensor pipe is busy 44 % of the time a CTA runs, at every size; the
-// apply takes 1.16 ms with sixteen epilogue warps and 1.31 ms with both halves' MMAs in turn and the levels drained in two
-// parts, so neither the drain's latency nor the dependence of consecutive MMAs is what is left.
+// One CTA: 128 rows of A (two row tiles) against 64 rows of B, all of K in 64-wide blocks.  Bound by the MMAs (28 digit pairs,
+// i + j <= 6: over a long row the dropped products stay far below the rounding of an FP64 chain, and the zero slices that
+// keep one shape per accumulator, oz_plan.cuh).  FP64 apply of three 16^3 elastic patterns (n_b = 4614, 256 right-hand
+// sides each, 32.7 GFLOP): 27.5 ms with FP64 FMAs, 0.97 ms so, and its error against 64 bits is the same (2.2e-10 of the
+// projected result, which is that of S^+).  The two groups of levels have an accumulator each (256 and 192 TMEM columns): one
+// is drained while the other is multiplied.  Drained levels are added into 91-bit integers per output (a 64-bit and a
+// 27-bit part): no FP64 operation before the final rounding.
 __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ OzGemmKernel P) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = smem;
-  uint8_t* sB = smem + G_RING * G_SLICE;
-  uint64_t* afull = reinterpret_cast<uint64_t*>(sB + OZ_TILE);   // [G_RING]
-  uint64_t* aempty = afull + G_RING;                             // [G_RING]
-  uint64_t* bfull = aempty + G_RING;                             // [2]
-  uint64_t* bempty = bfull + 2;                                  // [2]
-  uint64_t* tfull = bempty + 2;                                  // [2]
-  uint64_t* tempty = tfull + 2;                                  // [2]
+  uint8_t* sB = smem + OZ_RING * G_A + G_ZEROS;
+  uint64_t* afull = reinterpret_cast<uint64_t*>(sB + OZ_TILE);   // [OZ_RING], by slot
+  uint64_t* aempty = afull + OZ_RING;
+  uint64_t* bfull = aempty + OZ_RING;                            // [OZ_S], by slice
+  uint64_t* tfull = bfull + OZ_S;                                // [2], by group of levels
+  uint64_t* tempty = tfull + 2;
   uint64_t* done = tempty + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  volatile int* loads = abort_flag + 1;   // [3]: A slices, B halves 0 and 1 whose copies were issued
-  volatile int* seen = loads + 3;         // [3]: whose arrival the MMA thread has seen
+  volatile int* n_loads = abort_flag + 1;   // copies issued
 
   const OzGemm& G = P.G;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -98,24 +94,21 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
   const int nk = max(ke - kb, 0);
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < G_RING; ++i) {
-      mbar_init(&afull[i], 1);
-      mbar_init(&aempty[i], 1);
-    }
+    for (int i = 0; i < 2 * OZ_RING + OZ_S; ++i) mbar_init(&afull[i], 1);   // afull .. bfull
     for (int i = 0; i < 2; ++i) {
-      mbar_init(&bfull[i], 1);
-      mbar_init(&bempty[i], 1);
       mbar_init(&tfull[i], 1);
       mbar_init(&tempty[i], EPI_WARPS);
     }
     mbar_init(done, 1);
     *abort_flag = 0;
-    for (int i = 0; i < 3; ++i) loads[i] = seen[i] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  for (int i = threadIdx.x; i < G_ZEROS / 16; i += THREADS)   // never written again
+    *reinterpret_cast<uint4*>(sB - G_ZEROS + i * 16) = make_uint4(0, 0, 0, 0);
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // before the MMAs read them
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(2 * BUF_COLS));
+                 "r"(TMEM_COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   tc_fence_before();
@@ -124,122 +117,118 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0 && lane == 0) {
-    const uint8_t* A0 = G.A[p].tiles + (size_t)a0 * kt * OZ_TILE;
-    const uint8_t* A1 = G.A[p].tiles + (size_t)a1 * kt * OZ_TILE;
-    const uint8_t* B = G.B[p].tiles + (size_t)tn * kt * OZ_TILE;
+    const uint8_t* A0 = G.A[p].tiles + ((size_t)a0 * kt + kb) * OZ_TILE;
+    const uint8_t* A1 = G.A[p].tiles + ((size_t)a1 * kt + kb) * OZ_TILE;
+    const uint8_t* B = G.B[p].tiles + ((size_t)tn * kt + kb) * OZ_TILE;
     bool ok = true;
-    auto load_b = [&](int c, int h) {
-      if (c >= 1 && !(ok = mbar_wait(&bempty[h], (c & 1) ^ 1, abort_flag))) return;
-      mbar_expect_tx(&bfull[h], OZ_HALF);
-      bulk_load(sB + h * OZ_HALF, B + (size_t)(kb + c) * OZ_TILE + h * OZ_HALF, OZ_HALF, &bfull[h]);
-      loads[1 + h] = c + 1;
-    };
-    int g = 0;   // A slices so far
+    int last = -1;   // copies issued so far
     for (int c = 0; ok && c < nk; ++c) {
-      load_b(c, 0);
-      const size_t kofs = (size_t)(kb + c) * OZ_TILE;
-      for (int i = 0; ok && i < OZ_S; ++i, ++g) {
-        const int slot = g % G_RING, use = g / G_RING;
-        if (use >= 1 && !(ok = mbar_wait(&aempty[slot], (use & 1) ^ 1, abort_flag))) break;
-        mbar_expect_tx(&afull[slot], G_SLICE);
-        for (int q = 0; q < 4; ++q)
-          bulk_load(sA + slot * G_SLICE + q * OZ_SLICE_HALF,
-                    (q < 2 ? A0 : A1) + kofs + (q & 1) * OZ_HALF + i * OZ_SLICE_HALF, OZ_SLICE_HALF, &afull[slot]);
-        loads[0] = g + 1;
+      const size_t kofs = (size_t)c * OZ_TILE;
+#pragma unroll
+      for (int o = 0; o < OZ_LOADS; ++o) {
+        const OzLoad L = oz_load(o);
+        if (L.a >= 0) {
+          const int slot = oz_slot(c, oz_place(L.a)), use = oz_use(c, L.a);
+          if (use >= 1 && !(ok = mbar_wait(&aempty[slot], (use & 1) ^ 1, abort_flag))) break;
+          mbar_expect_tx(&afull[slot], G_A);
+          bulk_load(sA + slot * G_A, A0 + kofs + L.a * OZ_SLICE, OZ_SLICE, &afull[slot]);
+          bulk_load(sA + slot * G_A + OZ_SLICE, A1 + kofs + L.a * OZ_SLICE, OZ_SLICE, &afull[slot]);
+        } else {
+          // the MMA that gave up B's last slices also gave up A slice 0; those of the slices before were waited for with A
+          if (L.b == OZ_LOW && c >= 1 &&
+              !(ok = mbar_wait(&aempty[oz_slot(c - 1, oz_place(0))], oz_use(c - 1, 0) & 1, abort_flag)))
+            break;
+          mbar_expect_tx(&bfull[L.b], OZ_SLICE);
+          bulk_load(sB + L.b * OZ_SLICE, B + kofs + L.b * OZ_SLICE, OZ_SLICE, &bfull[L.b]);
+        }
+        last = c * OZ_LOADS + o;
       }
-      if (ok) load_b(c, 1);
     }
     if (!ok) {
       atomicCAS(G.error, 0, 21);
       *abort_flag = 1;
     }
+    *n_loads = last + 1;
   } else if (warp == 1 && lane == 0) {
     bool ok = true;
-    for (int c = 0; ok && c < nk; ++c)
-      for (int h = 0; ok && h < 2; ++h) {
-        ok = mbar_wait(&bfull[h], c & 1, abort_flag);
-        if (!ok) break;
-        seen[1 + h] = c + 1;
-        if (c >= 1 && !(ok = mbar_wait(&tempty[h], (c & 1) ^ 1, abort_flag))) break;
-        tc_fence_after();
-        const uint32_t acc = tmem + (uint32_t)(h * BUF_COLS);
-        const uint64_t bd = desc128(sB + h * OZ_HALF);
-        for (int i = 0; i < OZ_S; ++i) {
-          const int g = c * OZ_S + i, slot = g % G_RING;
-          if (h == 0) {
-            if (!(ok = mbar_wait(&afull[slot], (g / G_RING) & 1, abort_flag))) break;
-            seen[0] = g + 1;
-            tc_fence_after();
-          }
-          const uint64_t ad = desc128(sA + slot * G_SLICE);
-          const uint32_t id = idesc_bf16(32 * (OZ_S - i));
+    for (int c = 0; ok && c < nk; ++c) {
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) mma_f16(acc + 32 * i, ad + 2 * kk, bd + 2 * kk, id, (kk | i) ? 1u : 0u);
-          if (h == 1) mma_commit(&aempty[slot]);
-        }
-        if (!ok) break;
-        mma_commit(&tfull[h]);
-        mma_commit(&bempty[h]);
+      for (int q = 0; q < OZ_MMAS; ++q) {   // unrolled: the one thread's instructions are on the critical path
+        const OzMma M = oz_mma(q);
+        const int group = q < OZ_LOW ? 0 : 1;
+        const int slot = oz_slot(c, oz_place(M.a));
+        if (M.first && c >= 1 && !(ok = mbar_wait(&tempty[group], (c & 1) ^ 1, abort_flag))) break;
+        if ((group == 0 || M.a >= OZ_LOW) &&   // the block's first use of the slice
+            !(ok = mbar_wait(&afull[slot], oz_use(c, M.a) & 1, abort_flag)))
+          break;
+        if (M.new_b >= 0 && !(ok = mbar_wait(&bfull[M.new_b], c & 1, abort_flag))) break;
+        tc_fence_after();
+        const uint64_t ad = desc128(sA + slot * G_A), bd = desc128(sB + M.b * OZ_SLICE);
+        const uint32_t id = idesc_bf16(M.n);
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+          mma_f16(tmem + M.col, ad + 2 * kk, bd + 2 * kk, id, (kk || !M.first) ? 1u : 0u);
+        if (group == 1) mma_commit(&aempty[slot]);
+        if (q == OZ_LOW - 1) mma_commit(&tfull[0]);
       }
+      if (!ok) break;
+      mma_commit(&tfull[1]);
+    }
     if (!ok) {
       atomicCAS(G.error, 0, 22);
       *abort_flag = 1;
     }
     mma_commit(done);
   } else if (warp >= 2) {
-    const int quad = warp & 3, ch = (warp - 2) >> 2;
+    const int quad = warp & 3, c0 = ((warp - 2) >> 2) * EPI_COLS;
     const int row = quad * 32 + lane, i0 = tm * 128 + row;
-    long long hi[2][16];
-    uint32_t lo[2][16];
+    const uint32_t tbase = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)c0;
+    long long hi[EPI_COLS];
+    uint32_t lo[EPI_COLS];
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-      for (int q = 0; q < 16; ++q) {
-        hi[h][q] = 0;
-        lo[h][q] = 0;
-      }
+    for (int q = 0; q < EPI_COLS; ++q) {
+      hi[q] = 0;
+      lo[q] = 0;
+    }
     bool good = true;
     for (int c = 0; good && c < nk; ++c) {
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (good) {
-          good = __all_sync(0xffffffffu, mbar_wait(&tfull[h], c & 1, abort_flag));
-          if (!good) {
-            if (lane == 0) {
-              atomicCAS(G.error, 0, 23);
-              *abort_flag = 1;
-            }
-          } else {
-            tc_fence_after();
+      for (int group = 0; group < 2; ++group) {
+        if (!good) break;
+        good = __all_sync(0xffffffffu, mbar_wait(&tfull[group], c & 1, abort_flag));
+        if (!good) {
+          if (lane == 0) {
+            atomicCAS(G.error, 0, 23);
+            *abort_flag = 1;
+          }
+          break;
+        }
+        tc_fence_after();
+        const int l0 = group == 0 ? 0 : OZ_LOW, l1 = group == 0 ? OZ_LOW : OZ_S;
 #pragma unroll
-            for (int g = 0; g < 4; ++g) {
-              uint32_t v[OZ_S][4];
+        for (int g = 0; g < EPI_COLS / 8; ++g) {
+          uint32_t v[OZ_LOW][8];
 #pragma unroll
-              for (int s = 0; s < OZ_S; ++s) {
-                const uint32_t addr =
-                    tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(h * BUF_COLS + s * 32 + ch * 16 + g * 4);
-                asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-                             : "=r"(v[s][0]), "=r"(v[s][1]), "=r"(v[s][2]), "=r"(v[s][3])
-                             : "r"(addr));
-              }
-              asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-              if (g == 3) {
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&tempty[h]);
-              }
+          for (int l = l0; l < l1; ++l) tmem_ld8(v[l - l0], tbase + (uint32_t)(l * OZ_COLS + g * 8));
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          if (g == EPI_COLS / 8 - 1) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&tempty[group]);
+          }
 #pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                int d[OZ_S];
+          for (int q = 0; q < 8; ++q) {
+            int d[OZ_LOW];
 #pragma unroll
-                for (int s = 0; s < OZ_S; ++s) d[s] = __float2int_rn(__uint_as_float(v[s][q]));
-                long long& H = hi[h][g * 4 + q];
-                uint32_t& W = lo[h][g * 4 + q];
-                const long long l = (long long)d[4] * (1 << 18) + (long long)d[5] * (1 << 9) + ((long long)d[6] + W);
-                H += (long long)d[0] * (1 << 27) + (long long)d[1] * (1 << 18) + (long long)d[2] * (1 << 9) + d[3] +
-                     (l >> 27);
-                W = (uint32_t)l & ((1u << 27) - 1);
-              }
+            for (int l = 0; l < l1 - l0; ++l) d[l] = __float2int_rn(__uint_as_float(v[l][q]));
+            long long& X = hi[g * 8 + q];
+            uint32_t& W = lo[g * 8 + q];
+            if (group == 0) {
+              X += (long long)d[0] * (1 << 27) + (long long)d[1] * (1 << 18) + (long long)d[2] * (1 << 9) + d[3];
+            } else {
+              const long long l = (long long)d[0] * (1 << 18) + (long long)d[1] * (1 << 9) + ((long long)d[2] + W);
+              X += l >> 27;
+              W = (uint32_t)l & ((1u << 27) - 1);
             }
           }
         }
@@ -248,31 +237,34 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
     if (good && i0 < G.M[p]) {
       const int ea = G.A[p].exps[i0];
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int q = 0; q < 16; ++q) {
-          const int col = tn * 64 + h * 32 + ch * 16 + q;
-          if (col < G.N[p])
-            G.Z[p][(long long)col * G.ldz[p] + i0] =
-                rounded(hi[h][q], (long long)lo[h][q], 27, ea + G.B[p].exps[col] - 16 - 27);
-        }
+      for (int q = 0; q < EPI_COLS; ++q) {
+        const int col = tn * 64 + c0 + q;
+        if (col < G.N[p])
+          G.Z[p][(long long)col * G.ldz[p] + i0] = rounded(hi[q], (long long)lo[q], 27, ea + G.B[p].exps[col] - 16 - 27);
+      }
     }
   }
   __syncwarp();
   __syncthreads();
   if (threadIdx.x == 0) {
     if (!mbar_wait(done, 0)) atomicCAS(G.error, 0, 24);
-    if (*abort_flag) {   // copies issued but never waited for
-      for (int g = seen[0]; g < loads[0]; ++g) mbar_wait(&afull[g % G_RING], (g / G_RING) & 1);
-      for (int h = 0; h < 2; ++h)
-        for (int c = seen[1 + h]; c < loads[1 + h]; ++c) mbar_wait(&bfull[h], c & 1);
+    if (*abort_flag) {   // the last copy into every slot and slice, which nobody may have waited for
+      unsigned waited = 0;
+      for (int n = *n_loads - 1; n >= max(0, *n_loads - 2 * OZ_LOADS); --n) {
+        const int c = n / OZ_LOADS;
+        const OzLoad L = oz_load(n % OZ_LOADS);
+        const int bar = L.a >= 0 ? oz_slot(c, oz_place(L.a)) : 2 * OZ_RING + L.b;   // aempty lies between
+        if (waited >> bar & 1u) continue;
+        waited |= 1u << bar;
+        mbar_wait(&afull[bar], (L.a >= 0 ? oz_use(c, L.a) : c) & 1);
+      }
     }
   }
   __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * BUF_COLS));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS));
 }
 
 // Row exponents and slices of row-major operands, a CTA per (padded) row: the row is read twice, the second time from L1

@@ -9,18 +9,17 @@
 // would then round at 2^-52 of that value.  So a block is 28 bf16 MMAs (the pairs with i + j <= 6) into 7 accumulators;
 // the blocks are summed in integers and an output is rounded to FP64 once, where a chain of FMAs rounds at every term.
 //
-// A tile of 64 rows is stored as the 7 slices of its 64 x 64 digits in the layout the MMA reads (K-major rows of 128
-// bytes, 128-byte swizzle), rows 0-31 of all slices first, then rows 32-63: [half][slice][32][128 B], so that the
-// slices of a half are contiguous rows of one operand of N = 32 (7 - i) (slices 0 .. 6 - i against slice i).
+// A tile of 64 rows is stored as the 7 slices of its 64 x 64 digits, each in the layout the MMA reads (K-major rows of 128
+// bytes, 128-byte swizzle), so that consecutive slices are contiguous rows of one operand (which of them meet in an MMA:
+// oz_plan.cuh).
 #pragma once
 #include "common.cuh"
+#include "oz_plan.cuh"
 
 namespace fetirp {
 
-constexpr int OZ_S = 7, OZ_BITS = 9;
-constexpr int OZ_SLICE_HALF = 32 * 128;                      // 4 KB: 32 rows of one slice
-constexpr int OZ_HALF = OZ_S * OZ_SLICE_HALF;                // 28 KB: the slices of 32 rows
-constexpr int OZ_TILE = 2 * OZ_HALF;                         // 56 KB: one 64 x 64 tile
+constexpr int OZ_SLICE = 64 * 128;                           // 8 KB: 64 rows of one slice
+constexpr int OZ_TILE = OZ_S * OZ_SLICE;                     // 56 KB: one 64 x 64 tile
 constexpr int OZ_E_ZERO = -8000;                             // exponent of a row of zeros
 constexpr int OZ_E_BAD = 100000;                             // of a row with an infinity or a NaN: its products are NaN
 
@@ -103,7 +102,7 @@ __device__ __forceinline__ uint32_t oz_bf16(int d) { return __float_as_uint((flo
 
 // Byte offset of digit (row, k) of slice s in a tile
 __device__ __forceinline__ int oz_offset(int row, int k, int s) {
-  return (row >> 5) * OZ_HALF + s * OZ_SLICE_HALF + (row & 31) * 128 + ((((k >> 3) ^ row) & 7) << 4) + (k & 7) * 2;
+  return s * OZ_SLICE + row * 128 + ((((k >> 3) ^ row) & 7) << 4) + (k & 7) * 2;
 }
 #endif
 
