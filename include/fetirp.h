@@ -182,7 +182,7 @@ void fetirp_destroy(fetirp_ctx ctx);
  *     number of zero pivots differs.
  *  *pattern_id receives the id (0, 1, ...).
  * Device memory: a dense FP64 factor of (n rounded up to 64)^2 doubles, L_S^{-1} and S^+ in FP64, S^dag in FP32
- * and as tf32 and bf16 pairs, and from n_b = 256 on the digit slices of S^+ for FP64 products (14 bytes per entry;
+ * and as tf32 and bf16 pairs, and from n_b = 256 on the digit slices of S^+ for FP64 products (16 bytes per entry;
  * from n_b = 1024 on those of L_S^{-1} and its transpose as well).  Patterns with n_b >= 1024 form the bf16 pair of S^dag on the tensor cores and
  * compute S^+ and the FP32 and tf32 forms of S^dag only on the first call that needs them (a solve, an apply
  * or fetirp_get_pattern in FP64, FP32 or TF32X3; that call waits for them): a BF16X3 solve needs none of them

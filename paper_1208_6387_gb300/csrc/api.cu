@@ -95,6 +95,7 @@ __global__ void k_unpermute_rotate(int n_dofs, int dpn, int npad, const double* 
 struct OzBuf {
   DBuf<uint8_t> slices;
   DBuf<int> exps;
+  DBuf<uint32_t> flags;   // right-hand sides: the outputs of one product that FMAs compute
   OzOperand operand(long long rows, long long cols) {
     slices.ensure((size_t)oz_tiles(rows, cols) * OZ_TILE);
     exps.ensure((size_t)round_up(rows, 64));
@@ -825,20 +826,23 @@ void set_factored(LocalProblem& LP, int p, const PatternData& P, double* W) {
 // Scratch slices of the right-hand sides of the sliced FP64 products: pattern p's tiles from tile_off[p], its exponents
 // from row_off[p].
 struct OzRhs {
-  long long tiles = 0, rows = 0;
-  long long tile_off[MAXP] = {}, row_off[MAXP] = {};
+  long long tiles = 0, rows = 0, words = 0;
+  long long tile_off[MAXP] = {}, row_off[MAXP] = {}, word_off[MAXP] = {};
   bool on[MAXP] = {};
   void add(int p, int n_b, int n_rhs) {
     on[p] = n_b >= OZ_LOCAL_MIN_NB && (long long)n_b * n_b * n_rhs >= OZ_LOCAL_MIN_FMAS;
     tile_off[p] = tiles;
     row_off[p] = rows;
+    word_off[p] = words;
     if (!on[p]) return;
     tiles += oz_tiles(n_rhs, n_b);
     rows += round_up(n_rhs, 64);
+    words += oz_flag_words(n_b, n_rhs);
   }
   void ensure(OzBuf& b) const {
     b.slices.ensure((size_t)tiles * OZ_TILE);
     b.exps.ensure((size_t)rows);
+    b.flags.ensure((size_t)words);
   }
   OzOperand at(const OzBuf& b, int p) const { return {b.slices.p + (size_t)tile_off[p] * OZ_TILE, b.exps.p + row_off[p]}; }
 };
@@ -1368,10 +1372,14 @@ void local_f64(fetirp_ctx ctx, LocalProblem LP) {
   OzGemm G1, G2;
   OzSliceBatch B1, B2;
   G1.error = G2.error = ctx->tc_error.p;
-  auto add = [](OzGemm& G, const OzOperand& A, const OzOperand& B, int nb, int nr, int mode, double* Z, long long ld) {
+  // Z_p = A B_p, A(i, j) at a[i ai + j aj]
+  auto add = [&](OzGemm& G, int p, const OzOperand& A, const double* a, long long ai, long long aj, int mode,
+                 const double* b, double* Z) {
     const int i = G.n++;
-    G.A[i] = A; G.B[i] = B;
-    G.M[i] = G.K[i] = nb; G.N[i] = nr; G.mode[i] = mode; G.Z[i] = Z; G.ldz[i] = ld;
+    G.A[i] = A; G.B[i] = R.at(ctx->oz_rhs, p);
+    G.M[i] = G.K[i] = LP.n_b[p]; G.N[i] = LP.n_rhs[p]; G.mode[i] = mode; G.Z[i] = Z; G.ldz[i] = LP.ld[p];
+    G.a[i] = a; G.ai[i] = ai; G.aj[i] = aj; G.b[i] = b; G.ldb[i] = LP.ld[p];
+    G.flags[i] = ctx->oz_rhs.flags.p + R.word_off[p];
   };
   bool simt = false;
   for (int p = 0; p < LP.n_pat; ++p) {
@@ -1380,19 +1388,18 @@ void local_f64(fetirp_ctx ctx, LocalProblem LP) {
       continue;
     }
     const PatternData& P = *ctx->pats[p];
-    const OzOperand B = R.at(ctx->oz_rhs, p);
-    B1.add((const double*)LP.Y[p], LP.ld[p], LP.n_rhs[p], LP.n_b[p], 0, B);
-    if (LP.X[p]) add(G1, P.oz_lam.operand(), B, LP.n_b[p], LP.n_rhs[p], 1, LP.W[p], LP.ld[p]);
-    else add(G1, P.oz_S.operand(), B, LP.n_b[p], LP.n_rhs[p], 0, (double*)LP.Z[p], LP.ld[p]);
+    const double* Y = (const double*)LP.Y[p];
+    B1.add(Y, LP.ld[p], LP.n_rhs[p], LP.n_b[p], 0, R.at(ctx->oz_rhs, p));
+    if (LP.X[p]) add(G1, p, P.oz_lam.operand(), LP.X[p], 1, LP.ldx[p], 1, Y, LP.W[p]);   // Lam(i, j) at X[j ldx + i]
+    else add(G1, p, P.oz_S.operand(), (const double*)LP.S[p], LP.n_b[p], 1, 0, Y, (double*)LP.Z[p]);
   }
   oz_slice(B1, s);
   oz_gemm(G1, s);
   for (int p = 0; p < LP.n_pat; ++p) {
     if (!R.on[p]) continue;
     if (LP.X[p]) {
-      const OzOperand B = R.at(ctx->oz_rhs, p);
-      B2.add(LP.W[p], LP.ld[p], LP.n_rhs[p], LP.n_b[p], 0, B);
-      add(G2, ctx->pats[p]->oz_lamt.operand(), B, LP.n_b[p], LP.n_rhs[p], 2, (double*)LP.Z[p], LP.ld[p]);
+      B2.add(LP.W[p], LP.ld[p], LP.n_rhs[p], LP.n_b[p], 0, R.at(ctx->oz_rhs, p));
+      add(G2, p, ctx->pats[p]->oz_lamt.operand(), LP.X[p], LP.ldx[p], 1, 2, LP.W[p], (double*)LP.Z[p]);
     }
     LP.n_rhs[p] = 0;
   }

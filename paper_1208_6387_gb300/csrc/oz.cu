@@ -11,7 +11,7 @@ namespace {
 
 constexpr int THREADS = 320;                         // producer warp, MMA warp, 8 epilogue warps
 constexpr int EPI_WARPS = 8, EPI_COLS = OZ_COLS / (EPI_WARPS / 4);   // a warp's columns of its 32 rows
-constexpr int TMEM_COLS = 512;                       // 7 levels of 64 used
+constexpr int TMEM_COLS = 512;                       // 7 levels and the magnitudes, 64 each
 
 // K-major operand, 128-byte swizzle, 8-row groups 1024 bytes apart
 __device__ __forceinline__ uint64_t desc128(const void* p) {
@@ -24,26 +24,25 @@ __device__ __forceinline__ uint32_t idesc_bf16(int n) {
 }
 
 // v 2^q in FP64, rounded to nearest (halves away from zero), by integer operations: on this GPU an FP64 conversion or
-// addition costs more than this whole routine on the integer pipe.
-__device__ __forceinline__ double scaled_i64(long long v, int q) {
+// addition costs more than this whole routine on the integer pipe.  normal: the result is zero or a normal number.
+__device__ __forceinline__ double scaled_i64(long long v, int q, bool* normal) {
   const bool neg = v < 0;
   unsigned long long a = neg ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  *normal = true;
   if (a == 0) return 0.0;
   const int n = __clzll((long long)a);
   a <<= n;
   const int be = 1023 + 63 + q - n;
-  unsigned long long r = ((unsigned long long)(uint32_t)(be - 1) << 52) + (a >> 11) + ((a >> 10) & 1ull);
-  if (be <= 0) r = 0;
-  else if (be >= 2047) r = 0x7FF0000000000000ull;
+  *normal = be >= 1 && be <= 2045;
+  const unsigned long long r = ((unsigned long long)(uint32_t)(be - 1) << 52) + (a >> 11) + ((a >> 10) & 1ull);
   return __longlong_as_double((long long)(r | (neg ? 1ull << 63 : 0ull)));
 }
 
 // (hi + lo 2^-w) 2^e in FP64, one rounding after at least 62 significant bits; |lo| < 2^(w + 17)
-__device__ __forceinline__ double rounded(long long hi, long long lo, int w, int e) {
-  if (e > OZ_E_BAD / 2) return __longlong_as_double(0x7FF8000000000000ll);
+__device__ __forceinline__ double rounded(long long hi, long long lo, int w, int e, bool* normal) {
   const long long ah = hi < 0 ? -hi : hi;
   const int room = min(w, __clzll(ah) - 2);   // as many of lo's bits as hi leaves room for
-  return scaled_i64((hi << room) + (lo >> (w - room)), e - room);
+  return scaled_i64((hi << room) + (lo >> (w - room)), e - room, normal);
 }
 
 constexpr int G_A = 2 * OZ_SLICE;                       // an A slice of 128 rows: 16 KB
@@ -59,9 +58,8 @@ struct OzGemmKernel {
 }  // namespace
 
 // One CTA: 128 rows of A (two row tiles) against 64 rows of B, all of K in 64-wide blocks.  Bound by the MMAs (28 digit pairs,
-// i + j <= 6: over a long row the dropped products stay far below the rounding of an FP64 chain, and the zero slices that
-// keep one shape per accumulator, oz_plan.cuh).  FP64 apply of three 16^3 elastic patterns (n_b = 4614, 256 right-hand
-// sides each, 32.7 GFLOP): 27.5 ms with FP64 FMAs, 0.97 ms so, and its error against 64 bits is the same (2.2e-10 of the
+// the magnitudes, and the zero slices that keep one shape per accumulator, oz_plan.cuh).  FP64 apply of three 16^3 elastic patterns (n_b = 4614, 256 right-hand
+// sides each, 32.7 GFLOP): 27.5 ms with FP64 FMAs, 1.07 ms so (0.97 without the magnitudes), and its error against 64 bits is the same (2.2e-10 of the
 // projected result, which is that of S^+).  The two groups of levels have an accumulator each (256 and 192 TMEM columns): one
 // is drained while the other is multiplied.  Drained levels are added into 91-bit integers per output (a 64-bit and a
 // 27-bit part): no FP64 operation before the final rounding.
@@ -72,8 +70,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
   uint8_t* sB = smem + OZ_RING * G_A + G_ZEROS;
   uint64_t* afull = reinterpret_cast<uint64_t*>(sB + OZ_TILE);   // [OZ_RING], by slot
   uint64_t* aempty = afull + OZ_RING;
-  uint64_t* bfull = aempty + OZ_RING;                            // [OZ_S], by slice
-  uint64_t* tfull = bfull + OZ_S;                                // [2], by group of levels
+  uint64_t* bfull = aempty + OZ_RING;                            // [OZ_SLICES], by slice
+  uint64_t* tfull = bfull + OZ_SLICES;                           // [2], by group of levels
   uint64_t* tempty = tfull + 2;
   uint64_t* done = tempty + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
@@ -94,7 +92,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
   const int nk = max(ke - kb, 0);
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < 2 * OZ_RING + OZ_S; ++i) mbar_init(&afull[i], 1);   // afull .. bfull
+    for (int i = 0; i < 2 * OZ_RING + OZ_SLICES; ++i) mbar_init(&afull[i], 1);   // afull .. bfull
     for (int i = 0; i < 2; ++i) {
       mbar_init(&tfull[i], 1);
       mbar_init(&tempty[i], EPI_WARPS);
@@ -128,16 +126,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
       for (int o = 0; o < OZ_LOADS; ++o) {
         const OzLoad L = oz_load(o);
         if (L.a >= 0) {
-          const int slot = oz_slot(c, oz_place(L.a)), use = oz_use(c, L.a);
-          if (use >= 1 && !(ok = mbar_wait(&aempty[slot], (use & 1) ^ 1, abort_flag))) break;
+          const int slot = oz_slot(c, oz_place(L.a));   // every slot is used once a block
+          if (c >= 1 && !(ok = mbar_wait(&aempty[slot], (c & 1) ^ 1, abort_flag))) break;
           mbar_expect_tx(&afull[slot], G_A);
           bulk_load(sA + slot * G_A, A0 + kofs + L.a * OZ_SLICE, OZ_SLICE, &afull[slot]);
           bulk_load(sA + slot * G_A + OZ_SLICE, A1 + kofs + L.a * OZ_SLICE, OZ_SLICE, &afull[slot]);
         } else {
-          // the MMA that gave up B's last slices also gave up A slice 0; those of the slices before were waited for with A
-          if (L.b == OZ_LOW && c >= 1 &&
-              !(ok = mbar_wait(&aempty[oz_slot(c - 1, oz_place(0))], oz_use(c - 1, 0) & 1, abort_flag)))
-            break;
           mbar_expect_tx(&bfull[L.b], OZ_SLICE);
           bulk_load(sB + L.b * OZ_SLICE, B + kofs + L.b * OZ_SLICE, OZ_SLICE, &bfull[L.b]);
         }
@@ -155,11 +149,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
 #pragma unroll
       for (int q = 0; q < OZ_MMAS; ++q) {   // unrolled: the one thread's instructions are on the critical path
         const OzMma M = oz_mma(q);
-        const int group = q < OZ_LOW ? 0 : 1;
+        const int group = q < OZ_LOW ? 0 : 1;   // (the magnitudes are committed with the second one)
         const int slot = oz_slot(c, oz_place(M.a));
         if (M.first && c >= 1 && !(ok = mbar_wait(&tempty[group], (c & 1) ^ 1, abort_flag))) break;
         if ((group == 0 || M.a >= OZ_LOW) &&   // the block's first use of the slice
-            !(ok = mbar_wait(&afull[slot], oz_use(c, M.a) & 1, abort_flag)))
+            !(ok = mbar_wait(&afull[slot], c & 1, abort_flag)))
           break;
         if (M.new_b >= 0 && !(ok = mbar_wait(&bfull[M.new_b], c & 1, abort_flag))) break;
         tc_fence_after();
@@ -167,7 +161,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
         const uint32_t id = idesc_bf16(M.n);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          mma_f16(tmem + M.col, ad + 2 * kk, bd + 2 * kk, id, (kk || !M.first) ? 1u : 0u);
+          mma_f16(tmem + M.col, ad + 2 * kk, bd + 2 * kk, id, kk > 0 || (M.whole ? c > 0 : !M.first) ? 1u : 0u);
         if (group == 1) mma_commit(&aempty[slot]);
         if (q == OZ_LOW - 1) mma_commit(&tfull[0]);
       }
@@ -190,6 +184,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
       hi[q] = 0;
       lo[q] = 0;
     }
+    static_assert(EPI_COLS <= 32, "a bit per column");
+    uint32_t large = 0;   // columns with a level sum that FP32 may have rounded
     bool good = true;
     for (int c = 0; good && c < nk; ++c) {
 #pragma unroll
@@ -226,6 +222,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
             if (group == 0) {
               X += (long long)d[0] * (1 << 27) + (long long)d[1] * (1 << 18) + (long long)d[2] * (1 << 9) + d[3];
             } else {
+              const float top = fmaxf(fmaxf(fabsf(__uint_as_float(v[0][q])), fabsf(__uint_as_float(v[1][q]))),
+                                      fabsf(__uint_as_float(v[2][q])));
+              if (top >= 16777216.f) large |= 1u << (g * 8 + q);
               const long long l = (long long)d[0] * (1 << 18) + (long long)d[1] * (1 << 9) + ((long long)d[2] + W);
               X += l >> 27;
               W = (uint32_t)l & ((1u << 27) - 1);
@@ -234,14 +233,31 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
         }
       }
     }
-    if (good && i0 < G.M[p]) {
-      const int ea = G.A[p].exps[i0];
+    if (good) {
+      const bool in = i0 < G.M[p];
+      const int ea = G.A[p].exps[in ? i0 : 0];
+      const float line = sqrtf(64.f * nk) * 0x1p-8f;   // see oz.cuh
+      uint32_t word = 0;                               // lane q's: the rows of column q that FMAs compute
 #pragma unroll
-      for (int q = 0; q < EPI_COLS; ++q) {
-        const int col = tn * 64 + c0 + q;
-        if (col < G.N[p])
-          G.Z[p][(long long)col * G.ldz[p] + i0] = rounded(hi[q], (long long)lo[q], 27, ea + G.B[p].exps[col] - 16 - 27);
+      for (int g = 0; g < EPI_COLS / 8; ++g) {
+        uint32_t mag[8];
+        tmem_ld8(mag, tbase + (uint32_t)(OZ_S * OZ_COLS + g * 8));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int q = g * 8 + u, col = tn * 64 + c0 + q;
+          const int eb = G.B[p].exps[col];   // padded to 64 rows
+          bool normal;
+          const double z = rounded(hi[q], (long long)lo[q], 27, ea + eb - 16 - 27, &normal);
+          const bool zero = (ea == OZ_E_ZERO && eb != OZ_E_BAD) || (eb == OZ_E_ZERO && ea != OZ_E_BAD);
+          const bool fma_it = !zero && (!(__uint_as_float(mag[u]) >= line) || !normal || (large >> q & 1u));
+          const uint32_t rows = __ballot_sync(0xffffffffu, in && fma_it);
+          if (lane == q) word = rows;
+          if (in && col < G.N[p]) G.Z[p][(long long)col * G.ldz[p] + i0] = z;
+        }
       }
+      const int col = tn * 64 + c0 + lane, mw = (G.M[p] + 31) / 32, wr = tm * 4 + quad;
+      if (lane < EPI_COLS && col < G.N[p] && wr < mw) G.flags[p][(long long)col * mw + wr] = word;
     }
   }
   __syncwarp();
@@ -256,7 +272,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
         const int bar = L.a >= 0 ? oz_slot(c, oz_place(L.a)) : 2 * OZ_RING + L.b;   // aempty lies between
         if (waited >> bar & 1u) continue;
         waited |= 1u << bar;
-        mbar_wait(&afull[bar], (L.a >= 0 ? oz_use(c, L.a) : c) & 1);
+        mbar_wait(&afull[bar], c & 1);
       }
     }
   }
@@ -265,6 +281,104 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
   __syncthreads();
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS));
+}
+
+// The outputs that k_oz_gemm left to FMAs.  A thread per flag word looks for them (words of neighbouring threads lie a
+// grid apart, so that a flagged column or row spreads over the CTAs); the CTA's warps then take its words in turn: four rows
+// at a time and eight j where A's columns are contiguous (32 bytes a column), else row by row, 32 j.  Bound by the FP64 pipe.
+constexpr int FIX_THREADS = 256;
+struct OzFix {
+  OzGemm G;
+  long long word_off[OZ_MAXP + 1];
+};
+__global__ void __launch_bounds__(FIX_THREADS) k_oz_fix(const __grid_constant__ OzFix P) {
+  __shared__ int n_words;
+  __shared__ uint32_t todo[FIX_THREADS];      // flag words
+  __shared__ long long where[FIX_THREADS];    // and their indices
+  const OzGemm& G = P.G;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const long long total = P.word_off[G.n];
+  for (long long base = 0; base < total; base += (long long)gridDim.x * FIX_THREADS) {
+    const long long idx = base + blockIdx.x + (long long)gridDim.x * tid;
+    int p = 0;
+    if (tid == 0) n_words = 0;
+    __syncthreads();
+    if (idx < total) {
+      while (p + 1 < G.n && idx >= P.word_off[p + 1]) ++p;
+      const uint32_t w = G.flags[p][idx - P.word_off[p]];
+      if (w) {
+        const int at = atomicAdd(&n_words, 1);
+        todo[at] = w;
+        where[at] = idx;
+      }
+    }
+    __syncthreads();
+    const int n = n_words;
+    for (int it = tid >> 5; it < n; it += FIX_THREADS / 32) {
+      uint32_t w = todo[it];
+      const long long at = where[it];
+      p = 0;
+      while (p + 1 < G.n && at >= P.word_off[p + 1]) ++p;
+      const int M = G.M[p], K = G.K[p], mode = G.mode[p], mw = (M + 31) / 32;
+      const int c = (int)((at - P.word_off[p]) / mw), r0 = (int)((at - P.word_off[p]) % mw) * 32;
+      if (M - r0 < 32) w &= (1u << (M - r0)) - 1;   // set for real rows only, unless the product gave up
+      const double* b = G.b[p] + (long long)c * G.ldb[p];
+      double* z = G.Z[p] + (long long)c * G.ldz[p];
+      if (G.aj[p] != 1) {
+        const int jl = lane >> 2;
+        for (int g = 0; g < 32; g += 4) {
+          if (!(w >> g & 15u)) continue;
+          const int i = min(r0 + g + (lane & 3), M - 1);
+          const double* a = G.a[p] + i;
+          const int j0 = mode == 2 ? i : 0, j1 = mode == 1 ? i + 1 : K;
+          double s[4] = {0.0, 0.0, 0.0, 0.0};
+          for (int j = j0 + jl; j < j1; j += 32) {
+            double x[4], y[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const bool in = j + 8 * u < j1;
+              x[u] = in ? a[(long long)(j + 8 * u) * G.aj[p]] : 0.0;
+              y[u] = in ? b[j + 8 * u] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) s[u] = fma(x[u], y[u], s[u]);
+          }
+          double v = (s[0] + s[1]) + (s[2] + s[3]);
+#pragma unroll
+          for (int o = 16; o > 2; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          if (lane < 4 && (w >> (g + lane) & 1u)) z[i] = v;
+        }
+        continue;
+      }
+      while (w) {
+        const int i = r0 + __ffs(w) - 1;
+        w &= w - 1;
+        const double* a = G.a[p] + (long long)i * G.ai[p];
+        const int j0 = mode == 2 ? i : 0, j1 = mode == 1 ? i + 1 : K;
+        double s[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int j = j0 + lane; j < j1; j += 128)
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (j + 32 * u < j1) s[u] = fma(a[j + 32 * u], b[j + 32 * u], s[u]);
+        double v = (s[0] + s[1]) + (s[2] + s[3]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) z[i] = v;
+      }
+    }
+    __syncthreads();   // the list is read before the next one
+  }
+}
+
+// The digits and the magnitude of entry q of a group of eight, two entries a word
+__device__ __forceinline__ void put_entry(double x, int E, int q, uint32_t (&w)[OZ_SLICES][4]) {
+  int d[OZ_S];
+  oz_digits(x, E, d);
+#pragma unroll
+  for (int s = 0; s < OZ_SLICES; ++s) {
+    const uint32_t v = s == OZ_MAG ? oz_magnitude(x, E) : oz_bf16(d[s < OZ_S ? s : 0]);
+    w[s][q >> 1] = (q & 1) ? (w[s][q >> 1] | v << 16) : v;
+  }
 }
 
 // Row exponents and slices of row-major operands, a CTA per (padded) row: the row is read twice, the second time from L1
@@ -290,18 +404,15 @@ __global__ void __launch_bounds__(128) k_oz_slice(const __grid_constant__ OzSlic
   if (threadIdx.x == 0) P.out[p].exps[r] = E;
   uint8_t* out = P.out[p].tiles + (size_t)(r >> 6) * kt * OZ_TILE;
   for (int g = threadIdx.x; g < kt * 8; g += 128) {   // groups of 8 columns
-    uint32_t w[OZ_S][4];
+    uint32_t w[OZ_SLICES][4];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       const int c = g * 8 + q;
-      int d[OZ_S];
-      oz_digits(c >= c0 && c < c1 ? xr[c] : 0.0, E, d);
-#pragma unroll
-      for (int s = 0; s < OZ_S; ++s) w[s][q >> 1] = (q & 1) ? (w[s][q >> 1] | oz_bf16(d[s]) << 16) : oz_bf16(d[s]);
+      put_entry(c >= c0 && c < c1 ? xr[c] : 0.0, E, q, w);
     }
     uint8_t* o = out + (size_t)(g >> 3) * OZ_TILE;
 #pragma unroll
-    for (int s = 0; s < OZ_S; ++s)
+    for (int s = 0; s < OZ_SLICES; ++s)
       *reinterpret_cast<uint4*>(o + oz_offset(r & 63, (g & 7) * 8, s)) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
   }
 }
@@ -337,16 +448,11 @@ __global__ void __launch_bounds__(256) k_oz_slice_t(const double* __restrict__ x
   uint8_t* o = tiles + ((size_t)blockIdx.y * kt + blockIdx.x) * OZ_TILE;
   for (int u = threadIdx.x; u < 64 * 8; u += 256) {
     const int r = u & 63, k0 = (u >> 6) * 8, E = exps[r0 + r];
-    uint32_t w[OZ_S][4];
+    uint32_t w[OZ_SLICES][4];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      int d[OZ_S];
-      oz_digits(a[k0 + q][r], E, d);
+    for (int q = 0; q < 8; ++q) put_entry(a[k0 + q][r], E, q, w);
 #pragma unroll
-      for (int s = 0; s < OZ_S; ++s) w[s][q >> 1] = (q & 1) ? (w[s][q >> 1] | oz_bf16(d[s]) << 16) : oz_bf16(d[s]);
-    }
-#pragma unroll
-    for (int s = 0; s < OZ_S; ++s)
+    for (int s = 0; s < OZ_SLICES; ++s)
       *reinterpret_cast<uint4*>(o + oz_offset(r, k0, s)) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
   }
 }
@@ -395,13 +501,19 @@ void oz_slice_cols(const double* x, long long ld, int rows, int cols, int tri, c
 void oz_gemm(const OzGemm& G, cudaStream_t s) {
   oz_init();
   OzGemmKernel P;
+  OzFix F;
   P.G = G;
   int total = 0, n = 0;
+  long long words = 0;
   for (int p = 0; p < G.n; ++p) {
     if (G.M[p] <= 0 || G.N[p] <= 0) continue;
     P.G.A[n] = G.A[p]; P.G.B[n] = G.B[p];
     P.G.M[n] = G.M[p]; P.G.N[n] = G.N[p]; P.G.K[n] = G.K[p];
     P.G.mode[n] = G.mode[p]; P.G.Z[n] = G.Z[p]; P.G.ldz[n] = G.ldz[p];
+    P.G.a[n] = G.a[p]; P.G.ai[n] = G.ai[p]; P.G.aj[n] = G.aj[p];
+    P.G.b[n] = G.b[p]; P.G.ldb[n] = G.ldb[p]; P.G.flags[n] = G.flags[p];
+    F.word_off[n] = words;
+    words += oz_flag_words(G.M[p], G.N[p]);
     P.tiles_n[n] = ceil_div(G.N[p], 64);
     P.tile_off[n] = total;
     total += ceil_div(G.M[p], 128) * P.tiles_n[n];
@@ -411,6 +523,10 @@ void oz_gemm(const OzGemm& G, cudaStream_t s) {
   P.tile_off[n] = total;
   if (total == 0) return;
   k_oz_gemm<<<total, THREADS, G_SMEM, s>>>(P);
+  FETIRP_LAUNCH_CHECK();
+  F.G = P.G;
+  F.word_off[n] = words;
+  k_oz_fix<<<(unsigned)std::min<long long>((words + 7) / 8, 152 * 5), FIX_THREADS, 0, s>>>(F);
   FETIRP_LAUNCH_CHECK();
 }
 

@@ -5,11 +5,22 @@
 // digits of OZ_BITS bits, x = 2^E sum_s d_s 2^(-8 - 9 s), |d_s| <= 256: 63 bits below the row's scale, against the 53 of
 // an FP64 entry.  Digits up to 256 are exact in bf16, their products (<= 2^16) are exact, and the sums of one 64-wide
 // block of j over the s + 1 digit pairs of a level i + j = s are integers that FP32 holds exactly for levels 0 to 3
-// (<= 2^24); in levels 4 to 6 a sum beyond 2^24 would need some 300 products of one sign near their largest value, and
-// would then round at 2^-52 of that value.  So a block is 28 bf16 MMAs (the pairs with i + j <= 6) into 7 accumulators;
-// the blocks are summed in integers and an output is rounded to FP64 once, where a chain of FMAs rounds at every term.
+// (<= 2^24); a larger sum in levels 4 to 6 would need some 300 products of one sign near their largest value.
+// So a block is 28 digit pairs (those with i + j <= 6) on 7 levels; the blocks are summed in integers and an output is
+// rounded to FP64 once, where a chain of FMAs rounds at every term.
 //
-// A tile of 64 rows is stored as the 7 slices of its 64 x 64 digits, each in the layout the MMA reads (K-major rows of 128
+// What is dropped (an entry's bits below 2^-63 of its row's largest, the pairs beyond level 6) adds up to about
+// sqrt(n) 2^-63 2^(Ea + Eb) over n terms, whatever the entries; a chain of FMAs errs by 2e-17 to 2e-16 of sum |a||b|.  On
+// rows that are small where the other operand is large the scales say little about the sum, and there the chain is the
+// better one.  So the sum of |a||b| 2^-(Ea + Eb) is formed along with the digits (from magnitudes rounded down to bf16),
+// and an output where it is below sqrt(n) 2^-8 is computed by FP64 FMAs after all (k_oz_fix); so is one whose level sums
+// were too large, whose result is no normal number, or whose row holds an infinity or a NaN.  At that line the digits err by
+// 2e-17 of sum |a||b|, the chain by 4e-17 to 7e-17 (rms; rows that peak in one entry, rows graded against each other,
+// n = 256, 1158, 4614; below 2^-10 the chain is ahead).  On S^+ of 8^3 and 12^3 elastic and 64^2 heat patterns no output
+// falls below it: the smallest sums are 2^-4 sqrt(n), the digits err by 1e-18 there and the chain by 3e-17.  On the factors of
+// 12^3 16 % of the outputs of Lam = L_S^{-1} do (its rows peak at their diagonal) and 0.6 % of those of Lam^T.
+//
+// A tile of 64 rows is stored as the 7 slices of its 64 x 64 digits and their magnitudes, each in the layout the MMA reads (K-major rows of 128
 // bytes, 128-byte swizzle), so that consecutive slices are contiguous rows of one operand (which of them meet in an MMA:
 // oz_plan.cuh).
 #pragma once
@@ -19,9 +30,9 @@
 namespace fetirp {
 
 constexpr int OZ_SLICE = 64 * 128;                           // 8 KB: 64 rows of one slice
-constexpr int OZ_TILE = OZ_S * OZ_SLICE;                     // 56 KB: one 64 x 64 tile
+constexpr int OZ_TILE = OZ_SLICES * OZ_SLICE;                // 64 KB: one 64 x 64 tile
 constexpr int OZ_E_ZERO = -8000;                             // exponent of a row of zeros
-constexpr int OZ_E_BAD = 100000;                             // of a row with an infinity or a NaN: its products are NaN
+constexpr int OZ_E_BAD = 100000;                             // of a row with an infinity or a NaN
 
 // A sliced operand of `rows` x `cols`: ceil(rows / 64) x ceil(cols / 64) tiles, a row of tiles after the other, and an
 // exponent for every row (padded to 64).
@@ -57,8 +68,17 @@ struct OzGemm {
   int mode[OZ_MAXP];              // A(i, j): 0 dense, 1 zero for j > i, 2 zero for j < i
   double* Z[OZ_MAXP];             // Z[c * ldz + i]
   long long ldz[OZ_MAXP];
+  // the operands themselves, for the outputs that FMAs compute: A(i, j) at a[i * ai + j * aj] with ai or aj = 1, and
+  // B(c, j) at b[c * ldb + j]
+  const double* a[OZ_MAXP];
+  long long ai[OZ_MAXP], aj[OZ_MAXP];
+  const double* b[OZ_MAXP];
+  long long ldb[OZ_MAXP];
+  uint32_t* flags[OZ_MAXP];       // scratch: oz_flag_words(M, N) words, which outputs those are
   int* error = nullptr;
 };
+// A bit per output: word c ceil(M / 32) + i / 32
+inline long long oz_flag_words(long long M, long long N) { return (M + 31) / 32 * N; }
 void oz_gemm(const OzGemm& G, cudaStream_t s);
 
 // One-time kernel attribute set-up (large dynamic shared memory); call before any graph capture.
@@ -95,6 +115,13 @@ __device__ __forceinline__ void oz_digits(double x, int E, int (&d)[OZ_S]) {
     f = (f - q) >> 9;
   }
   d[0] = (int)f;
+}
+
+// bf16 bits of |x| 2^-E, rounded down (0 below 2^-126 and in rows with an infinity or a NaN)
+__device__ __forceinline__ uint32_t oz_magnitude(double x, int E) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ef = (int)(b >> 52) & 2047, f = ef - 1023 + 127 - E;
+  return ef == 0 || f <= 0 || E == OZ_E_BAD ? 0u : (uint32_t)f << 7 | ((uint32_t)(b >> 45) & 127u);
 }
 
 // bf16 bits of a digit (exact: |d| <= 256)

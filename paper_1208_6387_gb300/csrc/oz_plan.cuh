@@ -17,42 +17,50 @@ constexpr int OZ_COLS = 64;   // rows of B of a CTA: accumulator columns of a le
 // In a group i descends, so that the B slices are needed, and in the second group given up, from 0 on: the next block's are
 // loaded into their place meanwhile.
 constexpr int OZ_LOW = 4, OZ_PAD = 3;
-constexpr int OZ_MMAS = OZ_LOW + OZ_S;
+
+// Beside the digits a tile holds the magnitudes |x| 2^-E in bf16 as a slice of its own, OZ_MAG: one more MMA a block adds
+// sum |a||b| of every output over all blocks (what it is for: oz.cuh).
+constexpr int OZ_MAG = OZ_S, OZ_SLICES = OZ_S + 1;
+constexpr int OZ_MMAS = OZ_LOW + OZ_S + 1;
 
 struct OzMma {
   int a, b;      // A slice, first B slice
   int n, col;    // columns of the MMA (64 per B slice), first accumulator column
   bool first;    // the first of its accumulator in a block: it overwrites
+  bool whole;    // of an accumulator that is kept from block to block
   int new_b;     // B slice that no earlier MMA of the block reads (-1: none)
 };
 
-// MMA q of a block, in order of issue
+// A slices in order of issue: 3, 2, 1, 0 (levels 0 .. 3), then 6, 5, 4, the magnitudes, 3, 2, 1, 0 (levels 4 .. 6)
+constexpr int oz_mma_slice(int q) {
+  return q < OZ_LOW ? OZ_LOW - 1 - q : q < OZ_S ? OZ_S + OZ_LOW - 1 - q : q == OZ_S ? OZ_MAG : OZ_MMAS - 1 - q;
+}
 constexpr OzMma oz_mma(int q) {
   const bool low = q < OZ_LOW;
-  const int i = low ? OZ_LOW - 1 - q : OZ_MMAS - 1 - q;
+  const int i = oz_mma_slice(q);
+  if (i == OZ_MAG) return OzMma{OZ_MAG, OZ_MAG, OZ_COLS, OZ_COLS * OZ_S, false, true, OZ_MAG};
   const int l0 = low ? 0 : OZ_LOW, l1 = low ? OZ_LOW : OZ_S, top = l1 - 1 - i;
-  return OzMma{i, l0 - i, OZ_COLS * (l1 - l0), OZ_COLS * l0, top == 0, low || top >= OZ_LOW ? top : -1};
+  return OzMma{i, l0 - i, OZ_COLS * (l1 - l0), OZ_COLS * l0, top == 0, false, low || top >= OZ_LOW ? top : -1};
 }
 
-// Place of A slice i in the order of first use (3, 2, 1, 0, 6, 5, 4).  The A slices of a block sit in OZ_RING slots, each until
-// the second group's MMA of its slice; the first four are held meanwhile, the others pass through.  A block's first four
-// take the slots that the block before gives up first, those of its passing slices: slot = place, with its halves
-// exchanged in every other block.  use: how often the slot was used before.
-constexpr int OZ_RING = 8;
-constexpr int oz_place(int i) { return i < OZ_LOW ? OZ_LOW - 1 - i : OZ_LOW + OZ_S - 1 - i; }
+// Place of an A slice in the order of first use (3, 2, 1, 0, 6, 5, 4, magnitudes).  The A slices of a block sit in OZ_RING
+// slots, each until its last MMA of the block (the second group's, the magnitudes'); the first four are held meanwhile, the
+// others pass through.  A block's first four take the slots that the block before gives up first, those of its
+// passing slices: slot = place, with its halves exchanged in every other block.
+constexpr int OZ_RING = OZ_SLICES;
+constexpr int oz_place(int i) { return i < OZ_LOW ? OZ_LOW - 1 - i : i < OZ_S ? OZ_LOW + OZ_S - 1 - i : OZ_MAG; }
 constexpr int oz_slot(int block, int place) { return place ^ ((block & 1) * OZ_LOW); }
-constexpr int oz_use(int block, int i) { return oz_place(i) == OZ_LOW - 1 ? block >> 1 : block; }   // seven places of eight
 
-// Copies of a block in the order in which the block before gives up their places: A slice a, or B slice b.  B slices 0 to 3
-// follow the A slice whose slot the same MMA gave up, so that waiting for it is enough for them as well.
+// Copies of a block in the order in which the block before gives up their places: A slice a, or B slice b.  A B slice
+// follows the A slice whose slot the same MMA gave up, so that waiting for it is enough for both.
 struct OzLoad {
   int a, b;   // one of them, the other is -1
 };
-constexpr int OZ_LOADS = 2 * OZ_S;
+constexpr int OZ_LOADS = 2 * OZ_SLICES;
 constexpr OzLoad oz_load(int o) {
-  if (o < OZ_LOW) return OzLoad{OZ_LOW - 1 - o, -1};
-  if (o >= OZ_LOADS - OZ_LOW) return OzLoad{-1, o - (OZ_LOADS - OZ_S)};
-  return (o - OZ_LOW) % 2 ? OzLoad{OZ_S - 1 - (o - OZ_LOW) / 2, -1} : OzLoad{-1, (o - OZ_LOW) / 2};
+  constexpr int B = 16;
+  constexpr int order[OZ_LOADS] = {3, 2, 1, B + 0, 0, B + OZ_MAG, 6, B + 1, 5, B + 2, 4, B + 3, OZ_MAG, B + 4, B + 5, B + 6};
+  return order[o] < B ? OzLoad{order[o], -1} : OzLoad{-1, order[o] - B};
 }
 
 }  // namespace fetirp
