@@ -48,12 +48,14 @@ typedef enum {
 
 /* Arithmetic of the local multi-right-hand-side products S^+ Y (the hot contraction). */
 enum {
-  FETIRP_PREC_FP64 = 0, /* plain FP64 form */
+  FETIRP_PREC_FP64 = 0, /* plain FP64 form; large products by exact digit slices on the tensor cores, with FP64 FMAs for
+                           the outputs that the slices would hold worse (see fetirp_create_pattern) */
   FETIRP_PREC_FP32 = 1, /* FP32 products wrapped in FP64 outer refinement (defect correction) */
   FETIRP_PREC_TF32X3 = 2, /* tensor cores (tcgen05 kind::tf32), operands split hi+lo, 3 products, FP32
                              accumulation in TMEM; wrapped in FP64 outer refinement */
   FETIRP_PREC_AUTO = 3,   /* solves only (fetirp_options.precision): per structure, FP32 for latency-bound ones
-                             (every used pattern with n_b <= 512 and n_lambda <= 262144), TF32X3 otherwise; both inside the FP64 refinement */
+                             (every used pattern with n_b <= 512 and n_lambda <= 262144), TF32X3 otherwise; both inside the
+                             FP64 refinement */
   FETIRP_PREC_BF16X3 = 4  /* tensor cores (tcgen05 kind::f16 with bf16 operands, twice the tf32 rate), operands
                              split into bf16 pairs (16 significant bits), 3 products, FP32 accumulation in TMEM;
                              operator accurate to ~1e-5 relative; wrapped in FP64 outer refinement.  Rotations of
@@ -182,11 +184,14 @@ void fetirp_destroy(fetirp_ctx ctx);
  *     number of zero pivots differs.
  *  *pattern_id receives the id (0, 1, ...).
  * Device memory: a dense FP64 factor of (n rounded up to 64)^2 doubles, L_S^{-1} and S^+ in FP64, S^dag in FP32
- * and as tf32 and bf16 pairs, and from n_b = 256 on the digit slices of S^+ for FP64 products (16 bytes per entry;
- * from n_b = 1024 on those of L_S^{-1} and its transpose as well).  Patterns with n_b >= 1024 form the bf16 pair of S^dag on the tensor cores and
+ * and as tf32 and bf16 pairs.  Patterns with n_b >= 1024 form the bf16 pair of S^dag on the tensor cores and
  * compute S^+ and the FP32 and tf32 forms of S^dag only on the first call that needs them (a solve, an apply
  * or fetirp_get_pattern in FP64, FP32 or TF32X3; that call waits for them): a BF16X3 solve needs none of them
  * and applies S^+ in its FP64 refinement through L_S^{-1}.
+ * FP64 products of n_b >= 256 with n_b^2 times the right-hand sides >= 2^24 run on the tensor cores by digit slices of S^+
+ * (16 bytes per entry; of L_S^{-1} and its transpose, together as much, where S^+ is applied through them).  The
+ * first such product makes the slices and waits for them, later factorisations renew them; without memory for them, or
+ * when that product is being captured, it runs as FP64 FMAs.
  */
 fetirp_status fetirp_create_pattern(fetirp_ctx ctx, int32_t n_nodes, int32_t dofs_per_node,
                                     const int64_t* rowptr, const int32_t* col, const double* val,
@@ -334,9 +339,10 @@ fetirp_status fetirp_apply_block(fetirp_ctx ctx, int32_t k, const double* V, dou
 /* As fetirp_apply_block on DEVICE buffers; enqueued on the context's stream, returns without waiting, except
  * that the first call after a factorisation in FP64, FP32 or TF32X3 on a structure with a pattern of
  * n_b >= 1024 first forms that pattern's S^+ and FP32 / tf32 forms of S^dag (see fetirp_create_pattern) and
- * waits for them: make that call before any stream capture.  A bounded wait of the tensor-core pipeline
- * (FETIRP_PREC_TF32X3) that expired is reported only through fetirp_device_status, since the call returns
- * before the kernel has run. */
+ * waits for them: make that call before any stream capture.  The first large FP64 product waits for its digit
+ * slices as well (fetirp_create_pattern); captured before it, an apply is correct but runs on FP64 FMAs.  A bounded
+ * wait of the tensor-core pipeline (FETIRP_PREC_FP64, TF32X3 and BF16X3) that expired is reported only through
+ * fetirp_device_status, since the call returns before the kernel has run. */
 fetirp_status fetirp_apply_block_device(fetirp_ctx ctx, int32_t k, const double* d_V, double* d_Q,
                                         int32_t precision);
 

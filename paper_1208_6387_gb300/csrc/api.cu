@@ -96,8 +96,8 @@ struct OzBuf {
   DBuf<uint8_t> slices;
   DBuf<int> exps;
   DBuf<uint32_t> flags;   // right-hand sides: the outputs of one product that FMAs compute
-  OzOperand operand(long long rows, long long cols) {
-    slices.ensure((size_t)oz_tiles(rows, cols) * OZ_TILE);
+  OzOperand operand(long long rows, long long cols, int mode) {
+    slices.ensure((size_t)oz_tiles(rows, cols, mode) * OZ_TILE);
     exps.ensure((size_t)round_up(rows, 64));
     return {slices.p, exps.p};
   }
@@ -114,9 +114,10 @@ struct PatternData {
   DBuf<int64_t> d_rowptr;
   DBuf<int> d_col, d_newidx, zp;
   DBuf<double> d_val, L, diag0, S64, N, Nb, Dinv, LS, XS, DinvS, Sdag, Nwork;
-  // sliced operators of the FP64 local products (n_b >= OZ_LOCAL_MIN_NB): S^+ (with s64_ok), and of a pattern that may
-  // have no formed S^+ the factor Lam = L_S^{-1} and its transpose
+  // sliced operators of the FP64 local products: S^+, and of a pattern without a formed S^+ the factor Lam = L_S^{-1} and
+  // its transpose.  Made by the first product that takes them (ensure_slices) and from then on by every factorisation.
   OzBuf oz_S, oz_lam, oz_lamt;
+  bool oz_s_ok = false, oz_lam_ok = false;
   DBuf<int> zpS, d_zpiv;
   std::vector<int> h_zp;
   int* h_zp_pinned = nullptr;
@@ -515,6 +516,15 @@ constexpr long long OZ_LOCAL_MIN_FMAS = 1ll << 24;
 void form_splus64(PatternData& P, cudaStream_t s);
 void form_sdag64(PatternData& P, cudaStream_t s);
 
+void slice_splus(PatternData& P, cudaStream_t s) {
+  oz_slice_rows(P.S64.p, P.n_b, P.n_b, P.n_b, 0, P.oz_S.operand(P.n_b, P.n_b, 0), s);
+}
+void slice_lam(PatternData& P, cudaStream_t s) {
+  const int nb = P.n_b;
+  oz_slice_cols(P.XS.p, P.nbpad, nb, nb, 1, P.oz_lam.operand(nb, nb, 1), s);    // Lam(i, j) at XS[j nbpad + i]
+  oz_slice_rows(P.XS.p, P.nbpad, nb, nb, 2, P.oz_lamt.operand(nb, nb, 2), s);   // its transpose
+}
+
 void factor_stage_b(PatternData& P, int* tc_error, cudaStream_t s) {
   const int npad = P.npad, kd = P.kdim;
   // kernel: N_r = -K_rr^{-1} K_rz, N_z = I (right-hand side built on the host from the CSR)
@@ -558,7 +568,6 @@ void factor_stage_b(PatternData& P, int* tc_error, cudaStream_t s) {
   tile_inverses(P.LS.p, nbp, P.zpS.p, P.DinvS.p, s);
   tri_solve(P.LS.p, nbp, P.planS, P.zpS.p, P.XS.p, nbp, nbp, false, s, P.DinvS.p, true);   // X = L_S^{-1}
   const int nb = P.n_b;
-  if (nb >= OZ_LOCAL_MIN_NB) P.oz_S.operand(nb, nb);
   P.lds = round_up(nb, 4);
   P.ldsb = round_up(nb, 8);
   P.ld_y8 = P.ldsb;
@@ -587,8 +596,7 @@ void factor_stage_b(PatternData& P, int* tc_error, cudaStream_t s) {
   // the bf16 pair's own rounding (2^-17), not that of an FP32 rounding, so the FP32 and tf32 forms of S^dag
   // come from the FP64 S^+ (ensure_splus64).
   P.s64_ok = false;
-  oz_slice_cols(P.XS.p, nbp, nb, nb, -1, P.oz_lam.operand(nb, nb), s);   // Lam(i, j) at XS[j nbp + i]
-  oz_slice_rows(P.XS.p, nbp, nb, nb, 1, P.oz_lamt.operand(nb, nb), s);   // its transpose
+  if (P.oz_lam_ok) slice_lam(P, s);
   const double* A = nullptr;
   const double* E = nullptr;
   if (kd > 0) {
@@ -627,7 +635,7 @@ void form_splus64(PatternData& P, cudaStream_t s) {
   const int nb = P.n_b, nbp = P.nbpad, kd = P.kdim;
   const size_t nn = (size_t)nb * nb;
   lauum(P.XS.p, nbp, nbp, nb, P.S64.p, nb, s);   // S^+ = X^T X
-  if (nb >= OZ_LOCAL_MIN_NB) oz_slice_rows(P.S64.p, nb, nb, nb, 0, P.oz_S.operand(), s);
+  if (P.oz_s_ok) slice_splus(P, s);
   const double* Sdag = P.S64.p;
   if (kd > 0) {
     form_sdag64(P, s);
@@ -668,6 +676,34 @@ void ensure_splus64(PatternData& P, cudaStream_t s) {
   form_splus64(P, s);
   FETIRP_CUDA(cudaStreamSynchronize(s));
   P.s64_ok = true;
+}
+
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  FETIRP_CUDA(cudaStreamIsCapturing(s, &st));
+  return st != cudaStreamCaptureStatusNone;
+}
+
+// The sliced operator of pattern P's FP64 products (S^+, or Lam and its transpose where it is applied through them), made on
+// first use: 16 bytes an entry of S^+, as much for the two triangles together.  Blocks until made; patterns are shared by child
+// contexts, hence the lock.  False: not now (the stream is being captured, or there is no memory for them), and the caller
+// multiplies by FP64 FMAs.
+bool ensure_slices(PatternData& P, bool factored, cudaStream_t s) {
+  std::lock_guard<std::mutex> lock(P.s64_mu);
+  bool& ok = factored ? P.oz_lam_ok : P.oz_s_ok;
+  if (ok) return true;
+  if (capturing(s)) return false;
+  try {
+    if (factored) slice_lam(P, s);
+    else slice_splus(P, s);
+  } catch (const Error& e) {
+    if (e.status != FETIRP_ENOMEM) throw;
+    cudaGetLastError();
+    return false;
+  }
+  FETIRP_CUDA(cudaStreamSynchronize(s));
+  ok = true;
+  return true;
 }
 
 // The operators that products in precision prec read: everything but the bf16 pair needs ensure_splus64.
@@ -823,29 +859,67 @@ void set_factored(LocalProblem& LP, int p, const PatternData& P, double* W) {
   LP.W[p] = W;
 }
 
-// Scratch slices of the right-hand sides of the sliced FP64 products: pattern p's tiles from tile_off[p], its exponents
-// from row_off[p].
+// Which patterns of an FP64 product are multiplied sliced, and the scratch of their right-hand sides: pattern p's tiles from
+// tile_off[p], its exponents from row_off[p], the flags of its outputs from word_off[p].
 struct OzRhs {
   long long tiles = 0, rows = 0, words = 0;
   long long tile_off[MAXP] = {}, row_off[MAXP] = {}, word_off[MAXP] = {};
   bool on[MAXP] = {};
+  static bool large(int n_b, int n_rhs) {
+    return n_b >= OZ_LOCAL_MIN_NB && (long long)n_b * n_b * n_rhs >= OZ_LOCAL_MIN_FMAS;
+  }
   void add(int p, int n_b, int n_rhs) {
-    on[p] = n_b >= OZ_LOCAL_MIN_NB && (long long)n_b * n_b * n_rhs >= OZ_LOCAL_MIN_FMAS;
+    on[p] = true;
     tile_off[p] = tiles;
     row_off[p] = rows;
     word_off[p] = words;
-    if (!on[p]) return;
     tiles += oz_tiles(n_rhs, n_b);
     rows += round_up(n_rhs, 64);
     words += oz_flag_words(n_b, n_rhs);
   }
-  void ensure(OzBuf& b) const {
-    b.slices.ensure((size_t)tiles * OZ_TILE);
-    b.exps.ensure((size_t)rows);
-    b.flags.ensure((size_t)words);
+  // False as with ensure_slices
+  bool ensure(OzBuf& b, cudaStream_t s) const {
+    const size_t bytes = (size_t)tiles * OZ_TILE;
+    if (b.slices.n >= bytes && b.exps.n >= (size_t)rows && b.flags.n >= (size_t)words) return true;
+    if (capturing(s)) return false;
+    try {
+      b.slices.ensure(bytes);
+      b.exps.ensure((size_t)rows);
+      b.flags.ensure((size_t)words);
+    } catch (const Error& e) {
+      if (e.status != FETIRP_ENOMEM) throw;
+      cudaGetLastError();
+      return false;
+    }
+    return true;
   }
   OzOperand at(const OzBuf& b, int p) const { return {b.slices.p + (size_t)tile_off[p] * OZ_TILE, b.exps.p + row_off[p]}; }
 };
+
+// The sliced patterns of an FP64 product (LP: n_pat, n_rhs and which are factored), with their operators and scratch ready.
+OzRhs sliced_patterns(fetirp_ctx ctx, const LocalProblem& LP) {
+  OzRhs R;
+  for (int p = 0; p < LP.n_pat; ++p)
+    if (OzRhs::large(ctx->pats[p]->n_b, LP.n_rhs[p]) &&
+        ensure_slices(*ctx->pats[p], LP.X[p] != nullptr, ctx->stream))
+      R.add(p, ctx->pats[p]->n_b, LP.n_rhs[p]);
+  if (R.tiles > 0) {
+    ensure_tc_error(ctx);
+    if (!R.ensure(ctx->oz_rhs, ctx->stream)) R = OzRhs();
+  }
+  return R;
+}
+
+// Readies what the FP64 products of a block of k columns need beyond the operators, before any graph capture.
+void ensure_sliced(fetirp_ctx ctx, int k) {
+  LocalProblem LP{};
+  LP.n_pat = (int)ctx->pats.size();
+  for (int p = 0; p < LP.n_pat; ++p) {
+    LP.n_rhs[p] = (int)ctx->use[p].occs.size() * k;
+    set_factored(LP, p, *ctx->pats[p], nullptr);
+  }
+  sliced_patterns(ctx, LP);
+}
 
 void ensure_apply_buffers(fetirp_ctx ctx, int k) {
   long long total = 0, total8 = 0;
@@ -856,10 +930,6 @@ void ensure_apply_buffers(fetirp_ctx ctx, int k) {
   total = std::max(total, total8);   // the bf16 products use the FP32 buffers with leading dimension ld_y8
   ctx->Y64.ensure(total); ctx->Z64.ensure(total);
   if (factored_f64(ctx)) ctx->W64.ensure(total);
-  OzRhs R;
-  for (size_t p = 0; p < ctx->pats.size(); ++p)
-    R.add((int)p, ctx->pats[p]->n_b, (int)ctx->use[p].occs.size() * k);
-  R.ensure(ctx->oz_rhs);
   ctx->Y32.ensure(total); ctx->Z32.ensure(total); ctx->Ylo32.ensure(total);
   TcProblem T;   // would the tensor-core product split its reduction dimension?
   T.n_pat = (int)ctx->pats.size();
@@ -1361,14 +1431,11 @@ void project(fetirp_ctx ctx, double* V, int k, const double* in = nullptr) {   /
 // a formed S^+ (X[p]) goes through its factor, Lam^T (Lam Y), as two products.
 void local_f64(fetirp_ctx ctx, LocalProblem LP) {
   cudaStream_t s = ctx->stream;
-  OzRhs R;
-  for (int p = 0; p < LP.n_pat; ++p) R.add(p, LP.n_b[p], LP.n_rhs[p]);
+  const OzRhs R = sliced_patterns(ctx, LP);
   if (R.tiles == 0) {
     local_gemm_f64(LP, s);
     return;
   }
-  R.ensure(ctx->oz_rhs);
-  ensure_tc_error(ctx);
   OzGemm G1, G2;
   OzSliceBatch B1, B2;
   G1.error = G2.error = ctx->tc_error.p;
@@ -2408,6 +2475,7 @@ fetirp_status run_solve(fetirp_ctx ctx, double* d_lambda, double* d_u, fetirp_st
   }
   // operators formed on first use count as set-up (factorisation phase), not as solve time
   ensure_operators(ctx, prec);
+  ensure_sliced(ctx, prec == FETIRP_PREC_FP64 ? ctx->k : 1);   // block iterations; initial residual and refinement
   cudaEvent_t e0, e1;
   FETIRP_CUDA(cudaEventCreate(&e0));
   FETIRP_CUDA(cudaEventCreate(&e1));

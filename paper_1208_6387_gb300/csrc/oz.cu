@@ -115,8 +115,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0 && lane == 0) {
-    const uint8_t* A0 = G.A[p].tiles + ((size_t)a0 * kt + kb) * OZ_TILE;
-    const uint8_t* A1 = G.A[p].tiles + ((size_t)a1 * kt + kb) * OZ_TILE;
+    const OzRow r0 = oz_row(G.mode[p], a0, kt), r1 = oz_row(G.mode[p], a1, kt);
+    const uint8_t* A0 = G.A[p].tiles + (size_t)(r0.begin + kb - r0.first) * OZ_TILE;
+    const uint8_t* A1 = G.A[p].tiles + (size_t)(r1.begin + kb - r1.first) * OZ_TILE;
     const uint8_t* B = G.B[p].tiles + ((size_t)tn * kt + kb) * OZ_TILE;
     bool ok = true;
     int last = -1;   // copies issued so far
@@ -389,10 +390,10 @@ __global__ void __launch_bounds__(128) k_oz_slice(const __grid_constant__ OzSlic
   __shared__ unsigned long long wmax[4];
   int p = 0;
   while (p + 1 < P.n && (int)blockIdx.x >= P.row_off[p + 1]) ++p;
-  const int r = (int)blockIdx.x - P.row_off[p], rows = P.rows[p], cols = P.cols[p], tri = P.tri[p];
+  const int r = (int)blockIdx.x - P.row_off[p], rows = P.rows[p], cols = P.cols[p], mode = P.mode[p];
   const int kt = (cols + 63) / 64;
   const bool live = r < rows;
-  const int c0 = live && tri > 0 ? r : 0, c1 = live ? (tri < 0 ? r + 1 : cols) : 0;
+  const int c0 = live && mode == 2 ? r : 0, c1 = live ? (mode == 1 ? r + 1 : cols) : 0;
   const double* xr = P.x[p] + (long long)r * P.ld[p];
   unsigned long long mx = 0;
   for (int c = c0 + threadIdx.x; c < c1; c += 128) mx = max(mx, oz_abs_bits(xr[c]));
@@ -402,15 +403,16 @@ __global__ void __launch_bounds__(128) k_oz_slice(const __grid_constant__ OzSlic
   __syncthreads();
   const int E = oz_row_exp(max(max(wmax[0], wmax[1]), max(wmax[2], wmax[3])));
   if (threadIdx.x == 0) P.out[p].exps[r] = E;
-  uint8_t* out = P.out[p].tiles + (size_t)(r >> 6) * kt * OZ_TILE;
-  for (int g = threadIdx.x; g < kt * 8; g += 128) {   // groups of 8 columns
+  const OzRow tr = oz_row(mode, r >> 6, kt);
+  uint8_t* out = P.out[p].tiles + (size_t)tr.begin * OZ_TILE;
+  for (int g = tr.first * 8 + threadIdx.x; g < tr.last * 8; g += 128) {   // groups of 8 columns
     uint32_t w[OZ_SLICES][4];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       const int c = g * 8 + q;
       put_entry(c >= c0 && c < c1 ? xr[c] : 0.0, E, q, w);
     }
-    uint8_t* o = out + (size_t)(g >> 3) * OZ_TILE;
+    uint8_t* o = out + (size_t)((g >> 3) - tr.first) * OZ_TILE;
 #pragma unroll
     for (int s = 0; s < OZ_SLICES; ++s)
       *reinterpret_cast<uint4*>(o + oz_offset(r & 63, (g & 7) * 8, s)) = make_uint4(w[s][0], w[s][1], w[s][2], w[s][3]);
@@ -418,14 +420,14 @@ __global__ void __launch_bounds__(128) k_oz_slice(const __grid_constant__ OzSlic
 }
 
 // Exponents of the rows of a transposed operand (element (r, c) at x[r + c * sc]): a thread per row, 8 column strips
-__global__ void __launch_bounds__(256) k_oz_exps_t(const double* __restrict__ x, long long sc, int rows, int cols, int tri,
+__global__ void __launch_bounds__(256) k_oz_exps_t(const double* __restrict__ x, long long sc, int rows, int cols, int mode,
                                                    int* exps) {
   __shared__ unsigned long long m[8][32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, r = blockIdx.x * 32 + lane;
   unsigned long long mx = 0;
   if (r < rows)
     for (int c = w; c < cols; c += 8)
-      if (tri == 0 || (tri > 0 ? c >= r : c <= r)) mx = max(mx, oz_abs_bits(x[r + (long long)c * sc]));
+      if (mode == 0 || (mode == 2 ? c >= r : c <= r)) mx = max(mx, oz_abs_bits(x[r + (long long)c * sc]));
   m[w][lane] = mx;
   __syncthreads();
   if (w == 0) {
@@ -435,17 +437,19 @@ __global__ void __launch_bounds__(256) k_oz_exps_t(const double* __restrict__ x,
 }
 
 // Slices of one 64 x 64 tile of a transposed operand through shared memory
-__global__ void __launch_bounds__(256) k_oz_slice_t(const double* __restrict__ x, long long sc, int rows, int cols, int tri,
+__global__ void __launch_bounds__(256) k_oz_slice_t(const double* __restrict__ x, long long sc, int rows, int cols, int mode,
                                                     uint8_t* tiles, const int* __restrict__ exps) {
   __shared__ double a[64][65];   // [column][row]
   const int kt = gridDim.x, r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
+  const OzRow tr = oz_row(mode, blockIdx.y, kt);
+  if ((int)blockIdx.x < tr.first || (int)blockIdx.x >= tr.last) return;
   for (int i = threadIdx.x; i < 64 * 64; i += 256) {
     const int r = r0 + (i & 63), c = c0 + (i >> 6);
-    const bool in = r < rows && c < cols && (tri == 0 || (tri > 0 ? c >= r : c <= r));
+    const bool in = r < rows && c < cols && (mode == 0 || (mode == 2 ? c >= r : c <= r));
     a[i >> 6][i & 63] = in ? x[r + (long long)c * sc] : 0.0;
   }
   __syncthreads();
-  uint8_t* o = tiles + ((size_t)blockIdx.y * kt + blockIdx.x) * OZ_TILE;
+  uint8_t* o = tiles + (size_t)(tr.begin + blockIdx.x - tr.first) * OZ_TILE;
   for (int u = threadIdx.x; u < 64 * 8; u += 256) {
     const int r = u & 63, k0 = (u >> 6) * 8, E = exps[r0 + r];
     uint32_t w[OZ_SLICES][4];
@@ -483,18 +487,18 @@ void oz_slice(const OzSliceBatch& batch, cudaStream_t s) {
   FETIRP_LAUNCH_CHECK();
 }
 
-void oz_slice_rows(const double* x, long long ld, int rows, int cols, int tri, const OzOperand& out, cudaStream_t s) {
+void oz_slice_rows(const double* x, long long ld, int rows, int cols, int mode, const OzOperand& out, cudaStream_t s) {
   OzSliceBatch P;
-  P.add(x, ld, rows, cols, tri, out);
+  P.add(x, ld, rows, cols, mode, out);
   oz_slice(P, s);
 }
 
-void oz_slice_cols(const double* x, long long ld, int rows, int cols, int tri, const OzOperand& out, cudaStream_t s) {
+void oz_slice_cols(const double* x, long long ld, int rows, int cols, int mode, const OzOperand& out, cudaStream_t s) {
   if (rows <= 0 || cols <= 0) return;
   const int rt = ceil_div(rows, 64), kt = ceil_div(cols, 64);
-  k_oz_exps_t<<<rt * 2, 256, 0, s>>>(x, ld, rows, cols, tri, out.exps);
+  k_oz_exps_t<<<rt * 2, 256, 0, s>>>(x, ld, rows, cols, mode, out.exps);
   FETIRP_LAUNCH_CHECK();
-  k_oz_slice_t<<<dim3(kt, rt), 256, 0, s>>>(x, ld, rows, cols, tri, out.tiles, out.exps);
+  k_oz_slice_t<<<dim3(kt, rt), 256, 0, s>>>(x, ld, rows, cols, mode, out.tiles, out.exps);
   FETIRP_LAUNCH_CHECK();
 }
 

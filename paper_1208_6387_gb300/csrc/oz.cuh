@@ -34,32 +34,49 @@ constexpr int OZ_TILE = OZ_SLICES * OZ_SLICE;                // 64 KB: one 64 x 
 constexpr int OZ_E_ZERO = -8000;                             // exponent of a row of zeros
 constexpr int OZ_E_BAD = 100000;                             // of a row with an infinity or a NaN
 
-// A sliced operand of `rows` x `cols`: ceil(rows / 64) x ceil(cols / 64) tiles, a row of tiles after the other, and an
-// exponent for every row (padded to 64).
-inline long long oz_tiles(long long rows, long long cols) { return ((rows + 63) / 64) * ((cols + 63) / 64); }
+// A sliced operand of `rows` x `cols`: its 64 x 64 tiles, a row of tiles after the other, and an exponent for every row
+// (padded to 64).  Mode 1 (2): square and zero above (below) the diagonal; a row of tiles then ends (begins) with the diagonal
+// tile of the second (first) of the two rows that a CTA multiplies together, which have equally many.
+struct OzRow {
+  long long begin;      // tiles before this row of tiles
+  int first, last;      // its tile columns [first, last)
+};
+__host__ __device__ inline OzRow oz_row(int mode, int row, int kt) {
+  const long long q = row >> 1, odd = row & 1;
+  if (mode == 1) {
+    const int w = kt < 2 * q + 2 ? kt : (int)(2 * q + 2);
+    return {2 * q * (q + 1) + odd * w, 0, w};
+  }
+  if (mode == 2) return {2 * q * kt - 2 * q * (q - 1) + odd * (kt - 2 * q), (int)(2 * q), kt};
+  return {(long long)row * kt, 0, kt};
+}
+inline long long oz_tiles(long long rows, long long cols, int mode = 0) {
+  const int kt = (int)((cols + 63) / 64);
+  const OzRow last = oz_row(mode, (int)((rows + 63) / 64) - 1, kt);
+  return last.begin + last.last - last.first;
+}
 struct OzOperand {
   uint8_t* tiles = nullptr;
   int* exps = nullptr;
 };
 
 constexpr int OZ_MAXP = 16;
-// Slices of row-major operands in one launch (element (r, c) at x[r ld + c]); with tri = 1 (-1) only c >= r (c <= r) is
-// read and the rest is zero.
+// Slices of row-major operands in one launch (element (r, c) at x[r ld + c]); in mode 1 (2) only c <= r (c >= r) is read.
 struct OzSliceBatch {
   int n = 0;
   const double* x[OZ_MAXP];
   long long ld[OZ_MAXP];
-  int rows[OZ_MAXP], cols[OZ_MAXP], tri[OZ_MAXP], row_off[OZ_MAXP];
+  int rows[OZ_MAXP], cols[OZ_MAXP], mode[OZ_MAXP], row_off[OZ_MAXP];
   OzOperand out[OZ_MAXP];
-  void add(const double* x_, long long ld_, int rows_, int cols_, int tri_, const OzOperand& o) {
-    x[n] = x_; ld[n] = ld_; rows[n] = rows_; cols[n] = cols_; tri[n] = tri_; out[n] = o;
+  void add(const double* x_, long long ld_, int rows_, int cols_, int mode_, const OzOperand& o) {
+    x[n] = x_; ld[n] = ld_; rows[n] = rows_; cols[n] = cols_; mode[n] = mode_; out[n] = o;
     ++n;
   }
 };
 void oz_slice(const OzSliceBatch& batch, cudaStream_t s);
-void oz_slice_rows(const double* x, long long ld, int rows, int cols, int tri, const OzOperand& out, cudaStream_t s);
+void oz_slice_rows(const double* x, long long ld, int rows, int cols, int mode, const OzOperand& out, cudaStream_t s);
 // The same of a column-major operand (element (r, c) at x[r + c ld]).
-void oz_slice_cols(const double* x, long long ld, int rows, int cols, int tri, const OzOperand& out, cudaStream_t s);
+void oz_slice_cols(const double* x, long long ld, int rows, int cols, int mode, const OzOperand& out, cudaStream_t s);
 
 struct OzGemm {
   int n = 0;                      // products in the launch

@@ -39,8 +39,7 @@ int t_eta(int n, int k, const double* W, const double* Q, const double* r, int d
 int t_oz(int M, int N, int K, int mode, int by_cols, const double* a, long long lda, const double* b, long long ldb,
          double* z, long long ldz, long long* n_fma) {
   return guarded([&] {
-    const int tri = mode == 1 ? -1 : mode == 2 ? 1 : 0;
-    DBuf<uint8_t> sa(oz_tiles(M, K) * OZ_TILE), sb(oz_tiles(N, K) * OZ_TILE);
+    DBuf<uint8_t> sa(oz_tiles(M, K, mode) * OZ_TILE), sb(oz_tiles(N, K) * OZ_TILE);
     DBuf<int> ea(round_up(M, 64)), eb(round_up(N, 64)), error(1);
     DBuf<uint32_t> flags(oz_flag_words(M, N));
     error.zero(nullptr);
@@ -50,8 +49,8 @@ int t_oz(int M, int N, int K, int mode, int by_cols, const double* a, long long 
     G.M[0] = M; G.N[0] = N; G.K[0] = K; G.mode[0] = mode; G.Z[0] = z; G.ldz[0] = ldz;
     G.a[0] = a; G.ai[0] = by_cols ? 1 : lda; G.aj[0] = by_cols ? lda : 1; G.b[0] = b; G.ldb[0] = ldb;
     G.flags[0] = flags.p; G.error = error.p;
-    if (by_cols) oz_slice_cols(a, lda, M, K, tri, G.A[0], nullptr);
-    else oz_slice_rows(a, lda, M, K, tri, G.A[0], nullptr);
+    if (by_cols) oz_slice_cols(a, lda, M, K, mode, G.A[0], nullptr);
+    else oz_slice_rows(a, lda, M, K, mode, G.A[0], nullptr);
     oz_slice_rows(b, ldb, N, K, 0, G.B[0], nullptr);
     oz_gemm(G, nullptr);
     int code = 0;
