@@ -508,9 +508,9 @@ void factor_check(PatternData& P) {
 // Patterns with at least this many boundary dofs form S^dag on the tensor cores (factor_stage_b)
 constexpr int TC_SDAG_MIN_NB = 1024;
 // FP64 local products with at least this many boundary dofs and FMAs are sliced tensor-core products (oz.cuh).  Where
-// the line lies (whole apply, FP64 FMAs against sliced, us): n_b 294, 108 right-hand sides (9.3M FMAs) 92 / 103; 654, 32
-// (13.7M) 115 / 118; 1158, 16 (21M) 153 / 148; 456, 108 (22M) 142 / 119; 888, 150 (118M) 333 / 177; 2598, 64 (432M)
-// 1388 / 267; 1158, 1440 (1.9G) 3778 / 428.
+// the line lies (whole apply, FP64 FMAs against sliced, us): n_b 294, 108 right-hand sides (9.3M FMAs) 85 / 102; 654, 32
+// (13.7M) 107 / 115; 1158, 16 (21M) 141 / 141; 456, 108 (22M) 135 / 115; 888, 150 (118M) 306 / 144; 2598, 64 (432M)
+// 1391 / 245; 1158, 1440 (1.9G) 3720 / 406.
 constexpr int OZ_LOCAL_MIN_NB = 256;
 constexpr long long OZ_LOCAL_MIN_FMAS = 1ll << 24;
 void form_splus64(PatternData& P, cudaStream_t s);

@@ -322,8 +322,8 @@ int eta_chunks(int n);
 int eta_partials(int n, int k, const double* W, const double* Q, const double* r, DBuf<double>& partial,
                  cudaStream_t s, bool ds, int* n_read);
 // C (m x k) = A (m x m) B (m x k), row-major, FP64, one warp per row (small coarse products).
-// part (optional, small_gemm_parts(m) * m * k doubles): the inner dimension is split over that many CTA rows
-// and the slices added in order (deterministic)
+// part (optional, SMALL_GEMM_MAX_PARTS * m * k doubles, also for small_gemm_ds, which cuts finer): the inner dimension is
+// split over up to that many CTA rows and the slices added in order (deterministic)
 constexpr int SMALL_GEMM_MAX_PARTS = 8;
 int small_gemm_parts(int m);
 void small_gemm(int m, int k, const double* A, const double* B, double* C, cudaStream_t s, double* part = nullptr);

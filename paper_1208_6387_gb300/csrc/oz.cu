@@ -58,11 +58,12 @@ struct OzGemmKernel {
 }  // namespace
 
 // One CTA: 128 rows of A (two row tiles) against 64 rows of B, all of K in 64-wide blocks.  Bound by the MMAs (28 digit pairs,
-// the magnitudes, and the zero slices that keep one shape per accumulator, oz_plan.cuh).  FP64 apply of three 16^3 elastic patterns (n_b = 4614, 256 right-hand
-// sides each, 32.7 GFLOP): 27.5 ms with FP64 FMAs, 1.07 ms so (0.97 without the magnitudes), and its error against 64 bits is the same (2.2e-10 of the
-// projected result, which is that of S^+).  The two groups of levels have an accumulator each (256 and 192 TMEM columns): one
-// is drained while the other is multiplied.  Drained levels are added into 91-bit integers per output (a 64-bit and a
-// 27-bit part): no FP64 operation before the final rounding.
+// the magnitudes, and the zero slices that keep one shape per accumulator, oz_plan.cuh) and the hand-over of the
+// accumulators.  FP64 apply of three 16^3 elastic patterns (n_b = 4614, 256 right-hand sides each, 32.7 GFLOP): 27.5 ms with
+// FP64 FMAs, 1.08 ms so (0.97 without the magnitudes; this kernel 0.86), and its error against 64 bits is the same
+// (2.2e-10 of the projected result, which is that of S^+).  The two groups of levels have an accumulator each (256 and 192
+// TMEM columns): one is drained while the other is multiplied.  Drained levels are added into 91-bit integers per
+// output (a 64-bit and a 27-bit part): no FP64 operation before the final rounding.
 __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ OzGemmKernel P) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -286,7 +287,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
 
 // The outputs that k_oz_gemm left to FMAs.  A thread per flag word looks for them (words of neighbouring threads lie a
 // grid apart, so that a flagged column or row spreads over the CTAs); the CTA's warps then take its words in turn: four rows
-// at a time and eight j where A's columns are contiguous (32 bytes a column), else row by row, 32 j.  Bound by the FP64 pipe.
+// at a time and eight j where A's columns are contiguous (32 bytes a column), else row by row, 32 j.  Bound by the FP64 pipe
+// where there are any (a sixth of Lam Y on three 16^3 patterns, 64 right-hand sides each: 1.2 ms a product; 4.7 ms on
+// whole words, 6.6 on fewer CTAs), else by its launch (4 us).
 constexpr int FIX_THREADS = 256;
 struct OzFix {
   OzGemm G;
@@ -385,7 +388,7 @@ __device__ __forceinline__ void put_entry(double x, int E, int q, uint32_t (&w)[
 // Row exponents and slices of row-major operands, a CTA per (padded) row: the row is read twice, the second time from L1
 // or L2, and written as 16-byte groups of 8 digits of a slice.  Bound by latency and the integer digits, so every row
 // of every operand gets a CTA in one launch (a warp per row, a launch per operand: 39 us for 256 rows of 4614; this:
-// 27 us for all 768).
+// 28 us for all 768).
 __global__ void __launch_bounds__(128) k_oz_slice(const __grid_constant__ OzSliceBatch P) {
   __shared__ unsigned long long wmax[4];
   int p = 0;
