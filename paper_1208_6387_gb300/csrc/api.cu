@@ -877,13 +877,15 @@ struct OzRhs {
     rows += round_up(n_rhs, 64);
     words += oz_flag_words(n_b, n_rhs);
   }
+  bool fits(const OzBuf& b) const {
+    return b.slices.n >= (size_t)tiles * OZ_TILE && b.exps.n >= (size_t)rows && b.flags.n >= (size_t)words;
+  }
   // False as with ensure_slices
   bool ensure(OzBuf& b, cudaStream_t s) const {
-    const size_t bytes = (size_t)tiles * OZ_TILE;
-    if (b.slices.n >= bytes && b.exps.n >= (size_t)rows && b.flags.n >= (size_t)words) return true;
+    if (fits(b)) return true;
     if (capturing(s)) return false;
     try {
-      b.slices.ensure(bytes);
+      b.slices.ensure((size_t)tiles * OZ_TILE);
       b.exps.ensure((size_t)rows);
       b.flags.ensure((size_t)words);
     } catch (const Error& e) {
@@ -897,7 +899,9 @@ struct OzRhs {
 };
 
 // The sliced patterns of an FP64 product (LP: n_pat, n_rhs and which are factored), with their operators and scratch ready.
-OzRhs sliced_patterns(fetirp_ctx ctx, const LocalProblem& LP) {
+// Scratch that has to grow grows to the product of block_k columns, so that no narrower one, a captured one least of all,
+// sees it move again.
+OzRhs sliced_patterns(fetirp_ctx ctx, const LocalProblem& LP, int block_k) {
   OzRhs R;
   for (int p = 0; p < LP.n_pat; ++p)
     if (OzRhs::large(ctx->pats[p]->n_b, LP.n_rhs[p]) &&
@@ -905,7 +909,14 @@ OzRhs sliced_patterns(fetirp_ctx ctx, const LocalProblem& LP) {
       R.add(p, ctx->pats[p]->n_b, LP.n_rhs[p]);
   if (R.tiles > 0) {
     ensure_tc_error(ctx);
-    if (!R.ensure(ctx->oz_rhs, ctx->stream)) R = OzRhs();
+    if (!R.fits(ctx->oz_rhs)) {
+      OzRhs B;
+      for (int p = 0; p < LP.n_pat; ++p) {
+        const int n = std::max(LP.n_rhs[p], (int)ctx->use[p].occs.size() * block_k);
+        if (OzRhs::large(ctx->pats[p]->n_b, n)) B.add(p, ctx->pats[p]->n_b, n);
+      }
+      if (!B.ensure(ctx->oz_rhs, ctx->stream) && !R.ensure(ctx->oz_rhs, ctx->stream)) R = OzRhs();
+    }
   }
   return R;
 }
@@ -918,7 +929,7 @@ void ensure_sliced(fetirp_ctx ctx, int k) {
     LP.n_rhs[p] = (int)ctx->use[p].occs.size() * k;
     set_factored(LP, p, *ctx->pats[p], nullptr);
   }
-  sliced_patterns(ctx, LP);
+  sliced_patterns(ctx, LP, k);
 }
 
 void ensure_apply_buffers(fetirp_ctx ctx, int k) {
@@ -1431,7 +1442,7 @@ void project(fetirp_ctx ctx, double* V, int k, const double* in = nullptr) {   /
 // a formed S^+ (X[p]) goes through its factor, Lam^T (Lam Y), as two products.
 void local_f64(fetirp_ctx ctx, LocalProblem LP) {
   cudaStream_t s = ctx->stream;
-  const OzRhs R = sliced_patterns(ctx, LP);
+  const OzRhs R = sliced_patterns(ctx, LP, ctx->k);
   if (R.tiles == 0) {
     local_gemm_f64(LP, s);
     return;

@@ -288,8 +288,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_oz_gemm(const __grid_constant__ 
 // The outputs that k_oz_gemm left to FMAs.  A thread per flag word looks for them (words of neighbouring threads lie a
 // grid apart, so that a flagged column or row spreads over the CTAs); the CTA's warps then take its words in turn: four rows
 // at a time and eight j where A's columns are contiguous (32 bytes a column), else row by row, 32 j.  Bound by the FP64 pipe
-// where there are any (a sixth of Lam Y on three 16^3 patterns, 64 right-hand sides each: 1.2 ms a product; 4.7 ms on
-// whole words, 6.6 on fewer CTAs), else by its launch (4 us).
+// where there are any (Lam and Lam^T on three 16^3 patterns, 64 right-hand sides each: 1.2 ms for both products; with the
+// line of oz.cuh at 2^-7 2.3 ms, and 6.5 ms on 109 CTAs that took whole words), else by its launch (4 us).
 constexpr int FIX_THREADS = 256;
 struct OzFix {
   OzGemm G;

@@ -70,6 +70,23 @@ def test_slices_come_with_the_first_product(structure):
     assert np.linalg.norm(Q - ref) <= 1e-10 * np.linalg.norm(ref)
 
 
+def test_narrower_products_leave_the_scratch_in_place(structure):
+    """The scratch of the first sliced product, a narrow one here, is that of the whole block: what a program captured at
+    any width stays valid."""
+    prob, V, ref = structure
+    mem = Allocator()
+    ctx = _context(prob, **mem.hooks)
+    try:
+        F.fetirp_apply_block(ctx, np.ascontiguousarray(V[:, :3]))   # 81 right-hand sides: just above the line
+        held = dict(mem.out)
+        for k in (8, 5, 3):
+            Q = F.fetirp_apply_block(ctx, np.ascontiguousarray(V[:, :k]))
+            assert np.linalg.norm(Q - ref[:, :k]) <= 1e-10 * np.linalg.norm(ref[:, :k])
+        assert mem.out == held
+    finally:
+        F.fetirp_destroy(ctx)
+
+
 def test_without_memory_for_the_slices(structure):
     prob, V, ref = structure
     nb = prob.patterns[0].n_b
